@@ -460,8 +460,8 @@ int itc_step(const itc_image* img, const itc_params* p, const float* fields, con
     L.stats = stats;
     L.absolute = (p->flags & ITC_FIELDS_ABSOLUTE) ? 1 : 0;
     L.final_eval = 0;
-    const int dims[3] = {img->H, img->W, img->ndim == 3 ? img->G : 1};
-    return cuda_status(launch_run(L, 1, M, dims, reinterpret_cast<cudaStream_t>(stream), img->ndim));
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    return cuda_status(launch_run(L, 1, M > kRunThreads, 1, M, s, img->ndim));
 }
 
 size_t itc_plan_bytes(int B) {
@@ -614,7 +614,8 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         for (int b = 0; b < B; ++b) ints[io++] = order[b];
     }
     // iterations: images with up to 16, 32 or 64 codebook vectors share a CTA (8, 4 or 2 of them,
-    // 16, 32 or 64 threads each), larger ones have a CTA each; per dimension, the groups are
+    // 16, 32 or 64 threads each), those of up to kRunThreads have a CTA each and larger ones a
+    // cluster (listed first); per dimension, the groups are
     // listed by the pair work (iters x M^2) of their costliest image, largest first, so that the
     // long ones do not start last
     const int run_off = io;
@@ -624,12 +625,15 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
             if (descs[b].ndim == nd) order.push_back(b);
         auto cost = [&](int b) { return (double)(descs[b].iters + 1) * descs[b].M * descs[b].M; };
         std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return cost(a) > cost(c); });
+        // images of more than kRunThreads vectors have a launch of their own
+        std::stable_partition(order.begin(), order.end(), [&](int b) { return descs[b].M > kRunThreads; });
         int open[4] = {-1, -1, -1, -1};   // the group each span class is filling (int offset)
-        int ng = 0;
+        int ng = 0, nl = 0;
         for (int b : order) {
             const int M = descs[b].M;
             const int cl = M <= 16 ? 0 : (M <= 32 ? 1 : (M <= 64 ? 2 : 3));
-            const int span = 16 << cl, cap = cl == 3 ? 1 : kRunThreads / span;
+            // few images: a CTA each, which leaves every image an SM of its own
+            const int span = 16 << cl, cap = cl == 3 || (int)order.size() <= kSoloImages ? 1 : kRunThreads / span;
             if (open[cl] < 0 || ints[open[cl]] == cap) {
                 open[cl] = io;
                 ints[io] = 0;
@@ -640,8 +644,10 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
             }
             int* g = ints + open[cl];
             g[2 + g[0]++] = b;
+            nl += M > kRunThreads;
         }
-        h->run_ngroups[nd - 2] = ng;
+        h->run_nlarge[nd - 2] = nl;
+        h->run_ngroups[nd - 2] = ng - nl;
     }
     h->nints = io;
     h->bwd_order_off = bwd_off;
@@ -974,6 +980,7 @@ int itc_run_iterate_range(const void* plan_host, const void* plan_dev, int b0, i
 static int iterate_images(const PlanHeader* h, const void* plan_dev, int b0, int b1, bool whole, float* W,
                           itc_stats* stats, const WsView& v, cudaStream_t s) {
     if (b1 == b0) return ITC_OK;
+    const ImageDesc* hdescs = reinterpret_cast<const ImageDesc*>(reinterpret_cast<const unsigned char*>(h) + h->desc_off);
     const unsigned char* pd = reinterpret_cast<const unsigned char*>(plan_dev);
     RunLaunch R;
     memset(&R, 0, sizeof(R));
@@ -991,14 +998,17 @@ static int iterate_images(const PlanHeader* h, const void* plan_dev, int b0, int
     const int* groups = reinterpret_cast<const int*>(pd + h->ints_off) + h->run_groups_off;
     for (int nd = 2; nd <= 3; ++nd) {
         if (!(h->ndim_mask & (1 << nd))) continue;
-        int ctas = b1 - b0;
+        int large = 0, ctas = b1 - b0, large_ctas = b1 - b0;
         if (grouped) {
-            // the 3-D groups follow the 2-D ones
-            R.groups = groups + (nd == 3 ? (size_t)h->run_ngroups[0] * kGroupInts : 0);
+            large = large_ctas = h->run_nlarge[nd - 2];
             ctas = h->run_ngroups[nd - 2];
+            R.groups = groups;
+        } else {
+            for (int b = b0; b < b1; ++b) large += hdescs[b].ndim == nd && hdescs[b].M > kRunThreads;
         }
-        const int rc = cuda_status(launch_run(R, ctas, h->max_M, h->max_dim, s, nd));
+        const int rc = cuda_status(launch_run(R, large_ctas, large, ctas, h->max_M, s, nd));
         if (rc) return rc;
+        if (grouped) groups += (size_t)(large + ctas) * kGroupInts;   // the 3-D groups follow
     }
     return ITC_OK;
 }

@@ -15,13 +15,14 @@ constexpr int kMaxTapsG = 2 * ITC_MAX_RADIUS_G + 1;
 constexpr int kMaxClasses = 16;     // distinct (sigma, trunc, flags, ndim, dtype) classes per plan
 constexpr int kThreads = 256;       // fields / backward CTA size
 constexpr int kTileW = 64;          // output columns per fields tile
-constexpr int kRunThreads = 128;    // codebook-iteration CTA size
+constexpr int kRunThreads = 128;    // codebook-iteration CTA size (images of more vectors: a cluster)
+constexpr int kSoloImages = 152;    // up to one image per SM of the GPU: iterated one per CTA
 // Iteration group record: image count n, span (threads per image: 16, 32, 64 or 128), then up to
 // kRunThreads / 16 image indices.  Images with M <= span share one CTA, span threads each.
 constexpr int kGroupMax = 8;
 constexpr int kGroupInts = 2 + kGroupMax;
-// Dynamic shared floats per codebook vector of the iteration and backward-codebook kernels:
-// w (3), a (1), D (3), s (1), E (3).
+// Dynamic shared floats per codebook vector of the backward-codebook kernel: w (3), a (1), D (3),
+// s (1), E (3).
 constexpr int kCodebookSmemFloats = 11;
 
 // Truncated, unnormalised 1-D Gaussian taps of one parameter class, computed on the host in
@@ -122,7 +123,8 @@ struct PlanHeader {
     int max_bwd_tiles;          // most backward pixel tiles of one image
     int bwd_order_off;          // offset (ints) of the backward image order (B ints, most tiles first)
     int run_groups_off;         // offset (ints) of the iteration groups (kGroupInts ints each)
-    int run_ngroups[2];         // iteration groups of the 2-D images, then of the 3-D images
+    int run_nlarge[2], run_ngroups[2];   // iteration groups: the 2-D images of more than kRunThreads
+                                // vectors (one per group), the other 2-D groups, then the same in 3-D
     long long tmap_off;         // bytes from plan start to CUtensorMap[B] (input tiles)
     long long pad_floats;       // sum H*fpitch (padded per-pixel layout)
     int has_recursive;          // some class computes its fields by recursion
@@ -180,6 +182,7 @@ struct RunLaunch {
     const int* groups;          // whole batch: the images of each CTA (kGroupInts ints a CTA), else
                                 // one image a CTA, img_base + blockIdx.x
     const int* img_status;      // per-image status words of the fields pass (plans) or nullptr
+    int with_large;             // the launch covers images of more than kRunThreads vectors (set there)
 };
 
 struct BackwardLaunch {
@@ -244,8 +247,10 @@ cudaError_t launch_fields3d(const FieldsLaunch& L, int ntiles, int R_u, int R_v,
 bool fields_tma_supported(int ndim, int Ru, int Rv);
 int fields_tma_box(int dtype, int R, int tile_h, int* box_w, int* box_h);
 cudaError_t launch_fields_tma(const FieldsLaunch& L, int ntiles, int R, int dtype, cudaStream_t s);
-// ndim: the lattice dimension of every image of the launch (2 or 3)
-cudaError_t launch_run(const RunLaunch& L, int nimg, int max_M, const int* max_dim, cudaStream_t s, int ndim);
+// The iterations (itc_run.cu) of one lattice dimension: nlarge images of more than kRunThreads
+// codebook vectors and the others.  With L.groups: large_ctas groups of the former, then ctas groups
+// of the others; else both are the range's image count.
+cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, cudaStream_t s, int ndim);
 cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
 cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
 cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, cudaStream_t s);
