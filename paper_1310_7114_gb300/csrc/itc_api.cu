@@ -461,7 +461,7 @@ int itc_step(const itc_image* img, const itc_params* p, const float* fields, con
     L.absolute = (p->flags & ITC_FIELDS_ABSOLUTE) ? 1 : 0;
     L.final_eval = 0;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    return cuda_status(launch_run(L, 1, M > kRunThreads, 1, M, s, img->ndim));
+    return cuda_status(launch_run(L, 1, M > kRunThreads, 1, M, 0.0, s, img->ndim));
 }
 
 size_t itc_plan_bytes(int B) {
@@ -645,6 +645,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
             int* g = ints + open[cl];
             g[2 + g[0]++] = b;
             nl += M > kRunThreads;
+            if (M > kRunThreads) h->run_work[nd - 2] = std::max(h->run_work[nd - 2], cost(b));
         }
         h->run_nlarge[nd - 2] = nl;
         h->run_ngroups[nd - 2] = ng - nl;
@@ -999,14 +1000,21 @@ static int iterate_images(const PlanHeader* h, const void* plan_dev, int b0, int
     for (int nd = 2; nd <= 3; ++nd) {
         if (!(h->ndim_mask & (1 << nd))) continue;
         int large = 0, ctas = b1 - b0, large_ctas = b1 - b0;
+        double work = 0.0;
         if (grouped) {
             large = large_ctas = h->run_nlarge[nd - 2];
+            work = h->run_work[nd - 2];
             ctas = h->run_ngroups[nd - 2];
             R.groups = groups;
         } else {
-            for (int b = b0; b < b1; ++b) large += hdescs[b].ndim == nd && hdescs[b].M > kRunThreads;
+            for (int b = b0; b < b1; ++b) {
+                const ImageDesc& d = hdescs[b];
+                if (d.ndim != nd || d.M <= kRunThreads) continue;
+                ++large;
+                work = std::max(work, (double)(d.iters + 1) * d.M * d.M);
+            }
         }
-        const int rc = cuda_status(launch_run(R, large_ctas, large, ctas, h->max_M, s, nd));
+        const int rc = cuda_status(launch_run(R, large_ctas, large, ctas, h->max_M, work, s, nd));
         if (rc) return rc;
         if (grouped) groups += (size_t)(large + ctas) * kGroupInts;   // the 3-D groups follow
     }

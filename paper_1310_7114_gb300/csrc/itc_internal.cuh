@@ -125,6 +125,7 @@ struct PlanHeader {
     int run_groups_off;         // offset (ints) of the iteration groups (kGroupInts ints each)
     int run_nlarge[2], run_ngroups[2];   // iteration groups: the 2-D images of more than kRunThreads
                                 // vectors (one per group), the other 2-D groups, then the same in 3-D
+    double run_work[2];         // most (iters + 1) M^2 of the former, per dimension
     long long tmap_off;         // bytes from plan start to CUtensorMap[B] (input tiles)
     long long pad_floats;       // sum H*fpitch (padded per-pixel layout)
     int has_recursive;          // some class computes its fields by recursion
@@ -249,8 +250,9 @@ int fields_tma_box(int dtype, int R, int tile_h, int* box_w, int* box_h);
 cudaError_t launch_fields_tma(const FieldsLaunch& L, int ntiles, int R, int dtype, cudaStream_t s);
 // The iterations (itc_run.cu) of one lattice dimension: nlarge images of more than kRunThreads
 // codebook vectors and the others.  With L.groups: large_ctas groups of the former, then ctas groups
-// of the others; else both are the range's image count.
-cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, cudaStream_t s, int ndim);
+// of the others; else both are the range's image count.  work: most (iters + 1) M^2 of a large image.
+cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, double work, cudaStream_t s,
+                       int ndim);
 cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
 cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
 cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, cudaStream_t s);

@@ -581,6 +581,7 @@ __device__ __forceinline__ void iterate_wide(const RunLaunch& L, int img, const 
 // ------------------------------------------------------------- one image of more than kRunThreads vectors
 constexpr int kLargeCluster = 8;        // most CTAs per image (the portable cluster size)
 constexpr size_t kMergedSmem = 30 * 1024;   // 7 CTAs per SM
+constexpr double kClusterWork = 1.5e5;      // pairs over all iterations of an image: about 20 us of one CTA
 __host__ __device__ constexpr int large_threads(bool split) { return split ? 256 : 128; }
 // Where a vector's position lies: split by the parity of k for half_sums, in pairs for pair_sums.
 template <bool SPLIT>
@@ -845,7 +846,7 @@ int cluster_size(int nlarge, int max_M, int sms) {
 }
 
 template <int ND>
-cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max_M, cudaStream_t s) {
+cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max_M, double work, cudaStream_t s) {
     cudaError_t e;
     size_t smem = 0;
     if (nlarge > 0) {
@@ -853,14 +854,18 @@ cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         const int csize = cluster_size(nlarge, max_M, sms);
-        smem = large_smem_floats(max_M, csize, ND) * sizeof(float);
-        // one CTA per large image whose shared memory still lets 7 CTAs share an SM: one launch for
-        // all, so that no SM idles between the two (2000 images of M 64, 128 and 256, 50 iterations: 1.09
-        // ms in two launches, 0.96 ms in one)
-        if (csize == 1 && smem <= kMergedSmem) {
+        // One launch for all, a CTA per large image, where their shared memory still lets 7 CTAs share
+        // an SM and clusters are not to be had (2000 images of M 64, 128 and 256, 50 iterations: 1.09
+        // ms in two launches, 0.96 ms in one) or would not repay the second launch's 7 us: a CTA alone
+        // takes about 0.13 ns per pair (101 images of M 34 to 136, no iterations: 17 and 12 us).
+        const size_t one = large_smem_floats(max_M, 1, ND) * sizeof(float);
+        const bool others = L.groups ? ctas > 0 : ctas > nlarge;
+        if (one <= kMergedSmem && (csize == 1 || (others && work < kClusterWork))) {
             L.with_large = 1;
+            smem = one;
             if (L.groups) ctas += large_ctas;   // their groups come first
         } else {
+            smem = large_smem_floats(max_M, csize, ND) * sizeof(float);
             auto k = csize > 1 ? run_large_kernel<ND, true> : run_large_kernel<ND, false>;
             if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
                 return e;
@@ -876,8 +881,8 @@ cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max
             cfg.attrs = at;
             cfg.numAttrs = 1;
             if ((e = cudaLaunchKernelEx(&cfg, k, L)) != cudaSuccess) return e;
+            if (!others) return cudaSuccess;
             if (L.groups) L.groups += (size_t)large_ctas * kGroupInts;
-            else if (nlarge == ctas) return cudaSuccess;   // a range of large images alone
             smem = 0;
         }
     }
@@ -888,9 +893,10 @@ cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max
 
 }  // namespace
 
-cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, cudaStream_t s, int ndim) {
-    return ndim == 3 ? launch_nd<3>(L, large_ctas, nlarge, ctas, max_M, s)
-                     : launch_nd<2>(L, large_ctas, nlarge, ctas, max_M, s);
+cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, double work, cudaStream_t s,
+                       int ndim) {
+    return ndim == 3 ? launch_nd<3>(L, large_ctas, nlarge, ctas, max_M, work, s)
+                     : launch_nd<2>(L, large_ctas, nlarge, ctas, max_M, work, s);
 }
 
 }  // namespace itc
