@@ -91,12 +91,17 @@ void fill_taps(float sigma, int R, float* g, float* dg) {
 constexpr double kRecAlpha[2] = {1.680, -0.6803}, kRecBeta[2] = {3.735, -0.2598};
 constexpr double kRecOmega[2] = {0.6318, 1.997}, kRecDecay[2] = {1.783, 1.723};
 
-void make_rec_coef(const float* sigma, RecCoef* rc) {
+void make_rec_coef(const float* sigma, const int* side, RecCoef* rc) {
     for (int a = 0; a < 2; ++a)
         for (int t = 0; t < 2; ++t) {
-            const double mag = exp(-kRecDecay[t] / (double)sigma[a]), ang = kRecOmega[t] / (double)sigma[a];
-            rc->zr[a][t] = (float)(mag * cos(ang));
-            rc->zi[a][t] = (float)(mag * sin(ang));
+            const double b = kRecDecay[t] / (double)sigma[a], ang = kRecOmega[t] / (double)sigma[a];
+            rc->zr[a][t] = (float)(exp(-b) * cos(ang));
+            rc->zi[a][t] = (float)(exp(-b) * sin(ang));
+            for (int k = 0; k < 5; ++k) {
+                const double n = (double)((side[a] + 31) / 32 * (1LL << k));
+                rc->pr[a][t][k] = (float)(exp(-b * n) * cos(ang * n));
+                rc->pi[a][t][k] = (float)(exp(-b * n) * sin(ang * n));
+            }
         }
     for (int t = 0; t < 2; ++t) {
         rc->cr[t] = (float)kRecAlpha[t];
@@ -146,9 +151,9 @@ void fill_desc(const itc_image* img, const itc_params* p, int M, ImageDesc* d) {
     const int th = tile_h_of(img->ndim);
     d->tiles_u = (img->H + th - 1) / th;
     d->tiles_v = (img->W + kTileW - 1) / kTileW;
-    if (p->flags & ITC_RECURSIVE) {   // one S_XX partial per 32 columns
+    if (p->flags & ITC_RECURSIVE) {   // one S_XX partial per 8 (long sides: 32) columns
         d->tiles_u = 1;
-        d->tiles_v = (img->W + 31) / 32;
+        d->tiles_v = rec_scans(img->H, img->W) ? (img->W + 7) / 8 : (img->W + 31) / 32;
     }
     d->tiles_g = img->ndim == 3 ? d->G : 1;   // 3-D tiles: one gray slice each
     d->plane_floats = (long long)d->G * img->H * d->fpitch;
@@ -171,8 +176,9 @@ void fill_desc(const itc_image* img, const itc_params* p, int M, ImageDesc* d) {
     if (p->flags & ITC_RECURSIVE) {
         float sw[3];
         for (int i = 0; i < 3; ++i) sw[i] = i < img->ndim ? self_width(p, i) : 1.f;
-        make_rec_coef(p->sigma, &d->rc);
-        make_rec_coef(sw, &d->rc_self);
+        const int side[2] = {img->H, img->W};
+        make_rec_coef(p->sigma, side, &d->rc);
+        make_rec_coef(sw, side, &d->rc_self);
     }
     d->self_tiles_u = d->tiles_u;
     d->self_off = -1;

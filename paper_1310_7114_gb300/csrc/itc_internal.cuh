@@ -44,7 +44,13 @@ struct Taps {
 struct RecCoef {
     float zr[2][2], zi[2][2];
     float cr[2], ci[2];
+    float pr[2][2][5], pi[2][2][5];   // z^(seg 2^k), seg = ceil(side / 32): a lane's share of a line
 };
+
+// Recursive fields of images with no side longer than this filter each line with a warp in shared
+// memory (three arrays of 8 lines: 201 KB); others run one sequential recursion per line.
+constexpr int kRecMaxLine = 2048;
+__host__ __device__ constexpr bool rec_scans(int H, int W) { return H <= kRecMaxLine && W <= kRecMaxLine; }
 
 // One image as the kernels see it (device-resident inside a plan, or passed by value).
 struct ImageDesc {

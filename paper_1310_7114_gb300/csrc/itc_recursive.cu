@@ -10,14 +10,27 @@
 //   g * x  = Re sum_t c_t (s0 + r0),     (d g) * x = Re sum_t c_t (r1 - s1)     (d = offset)
 // with zero states at the ends (no data outside the image), so the kernel is untruncated.
 //
-// Pass along v (one lane per row, rows staged through shared memory in 32 x 32 tiles so that
-// global accesses are coalesced; a warp per 32-row block, the blocks of an image spread over the
-// grid's y dimension): T = g_v * h, T_v = (d g)_v * h into two scratch planes (the causal part is
-// stored, the anticausal part added).  Pass along u (one thread per column, 128 columns per CTA,
-// so warps read and write whole row segments; rows in prefetched chunks): A = g_u * T,
-// F_u = (d g)_u * T, F_v = g_u * T_v into the field planes, same order; the column pass also sums
-// h A per column (FP64) and each warp's 32 columns into one S_XX partial, in a fixed order.  The
-// self-overlap pass (mode 1) computes A alone into the A_s plane with one scratch plane.
+// Lines of up to kRecMaxLine samples (rec_rows_scan, rec_cols_scan): a warp filters a line that lies in
+// shared memory, each lane a contiguous segment of it.  The recursions are linear, so a segment's
+// state is its own (from zero) plus the incoming state times a power of z:
+//   s0' = z^n s0 + b0,   s1' = z^n s1 + n z^n s0 + b1
+// Every lane runs its segment from zero for (b0, b1) of both directions, two warp scans carry the
+// states across the lanes (powers z^(L 2^k) from the plan), and a second run writes the outputs.
+// A line thus takes 4 L steps of a chain instead of 2 n, for 1.7 times the arithmetic.  A warp takes two
+// neighbouring lines at once as the halves of packed FP32 operations.  Pass along v: lines are image
+// rows, T = g_v * h, T_v = (d g)_v * h into two scratch planes.  Pass along u: a CTA takes 8 columns
+// (32-byte row pieces of the planes), A = g_u * T and F_u = (d g)_u * T, in a launch of its own
+// F_v = g_u * T_v; its h A sum is one S_XX partial (FP32 over 8 products, then FP64 in a fixed order).
+// What bounds it now is the memory round trips between a CTA's phases (8 to 12 warps per SM at 101 KB
+// of shared memory for 1024 samples): all loads of a phase are in flight together.
+// 48 images of 128 to 1024 px a side (15 Mpx), microseconds, before and now: along v 431 and 102, along u
+// 694 and 245, the self-overlap pass 361 and 60, 567 and 105.
+//
+// Longer lines keep one sequential recursion per row and column (rec_rows_kernel, rec_cols_kernel):
+// along v one lane per row, rows staged through shared memory in 32 x 32 tiles, the causal part
+// stored and the anticausal part added; along u one thread per column, 128 columns per CTA, rows in
+// prefetched chunks, one S_XX partial per 32 columns.
+// The self-overlap pass (mode 1) computes A alone into the A_s plane with one scratch plane.
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -36,6 +49,334 @@ __device__ __forceinline__ const ImageDesc& rec_image(const RecursiveLaunch& L) 
     return L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x)];
 }
 
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+
+// A complex number for each of two neighbouring lines, in packed halves.
+struct Cplx2 {
+    float2 r, i;
+};
+__device__ __forceinline__ float2 both(float a) { return f2(a, a); }
+// z s and z s + t, one z for both lines
+__device__ __forceinline__ Cplx2 cmul2(const Cplx& z, const Cplx2& s) {
+    return {__ffma2_rn(both(z.r), s.r, __fmul2_rn(both(-z.i), s.i)), __ffma2_rn(both(z.r), s.i, __fmul2_rn(both(z.i), s.r))};
+}
+__device__ __forceinline__ Cplx2 cfma2(const Cplx& z, const Cplx2& s, const Cplx2& t) {
+    return {__ffma2_rn(both(z.r), s.r, __ffma2_rn(both(-z.i), s.i, t.r)),
+            __ffma2_rn(both(z.r), s.i, __ffma2_rn(both(z.i), s.r, t.i))};
+}
+template <bool UP>
+__device__ __forceinline__ float shfl_by(float v, int o) {
+    return UP ? __shfl_up_sync(0xffffffffu, v, o) : __shfl_down_sync(0xffffffffu, v, o);
+}
+template <bool UP>
+__device__ __forceinline__ Cplx2 shfl_by(const Cplx2& s, int o) {
+    return {f2(shfl_by<UP>(s.r.x, o), shfl_by<UP>(s.r.y, o)), f2(shfl_by<UP>(s.i.x, o), shfl_by<UP>(s.i.y, o))};
+}
+
+constexpr int kRecPairs = 4;               // line pairs (warps) per CTA of the scan kernels
+constexpr int kRecLines = 2 * kRecPairs;
+
+// One axis of the recursion: z, the weights and z^(seg 2^k) of both terms.
+struct RecAxis {
+    Cplx z[2], c[2], zp[2][5];
+    __device__ __forceinline__ RecAxis(const RecCoef& rc, int a) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            z[t] = {rc.zr[a][t], rc.zi[a][t]};
+            c[t] = {rc.cr[t], rc.ci[t]};
+#pragma unroll
+            for (int k = 0; k < 5; ++k) zp[t][k] = {rc.pr[a][t][k], rc.pi[a][t][k]};
+        }
+    }
+};
+
+// States of the two terms: s0 (and, MOM, s1) of one direction.
+template <bool MOM>
+struct RecState {
+    Cplx2 s0[2], s1[MOM ? 2 : 1];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            s0[t] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+            s1[MOM ? t : 0] = s0[t];
+        }
+    }
+    // s1' = z s1 + z s0, s0' = z s0 + x: the state after sample x
+    __device__ __forceinline__ void causal(const RecAxis& A, float2 x) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const Cplx2 p = cmul2(A.z[t], s0[t]);
+            if constexpr (MOM) s1[t] = cfma2(A.z[t], s1[t], p);
+            s0[t] = {__fadd2_rn(p.r, x), p.i};
+        }
+    }
+    // r0' = z (r0 + x), r1' = z r1 + r0': the state one place to the left of sample x
+    __device__ __forceinline__ void anticausal(const RecAxis& A, float2 x) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            s0[t] = cmul2(A.z[t], Cplx2{__fadd2_rn(s0[t].r, x), s0[t].i});
+            if constexpr (MOM) s1[t] = cfma2(A.z[t], s1[t], s0[t]);
+        }
+    }
+    // acc + sign Re sum_t c_t s_t
+    static __device__ __forceinline__ float2 weigh(const RecAxis& A, const Cplx2* s, float sign, float2 acc) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+            acc = __ffma2_rn(both(sign * A.c[t].r), s[t].r, __ffma2_rn(both(-sign * A.c[t].i), s[t].i, acc));
+        return acc;
+    }
+    // the lanes' own states (from zero) become the states that enter their segments: inclusive scan,
+    // then one lane on.  UP: from the lower lanes (causal)
+    template <bool UP>
+    __device__ __forceinline__ void scan(const RecAxis& A, int seg) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const int o = 1 << k;
+            const float2 n = both((float)(seg * o));
+            const bool from = UP ? lane >= o : lane + o < 32;
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const Cplx zp = {from ? A.zp[t][k].r : 0.f, from ? A.zp[t][k].i : 0.f};   // 0: no lane there
+                const Cplx2 p = cmul2(zp, shfl_by<UP>(s0[t], o));
+                if constexpr (MOM) {
+                    s1[t] = cfma2(zp, shfl_by<UP>(s1[t], o), s1[t]);
+                    s1[t] = {__ffma2_rn(n, p.r, s1[t].r), __ffma2_rn(n, p.i, s1[t].i)};
+                }
+                s0[t] = {__fadd2_rn(s0[t].r, p.r), __fadd2_rn(s0[t].i, p.i)};
+            }
+        }
+        const bool none = UP ? lane == 0 : lane == 31;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            s0[t] = shfl_by<UP>(s0[t], 1);
+            if constexpr (MOM) s1[t] = shfl_by<UP>(s1[t], 1);
+        }
+        if (none) clear();
+    }
+};
+
+// The whole warp filters the two lines in x: seg samples per lane (zeros past the lines' end), lane
+// l's at x + l * str, str odd.  o0 = g * x and (MOM) o1 = (d g) * x in the same layout.
+template <bool MOM>
+__device__ __forceinline__ void filter_lines(const RecAxis& A, const float2* x, float2* o0, float2* o1, int seg, int str) {
+    const int lane = threadIdx.x & 31;
+    x += lane * str;
+    o0 += lane * str;
+    o1 += lane * str;
+    RecState<MOM> s, r;
+    s.clear();
+    r.clear();
+    // (1) each segment from zero, both directions side by side
+#pragma unroll 2
+    for (int j = 0; j < seg; ++j) {
+        s.causal(A, x[j]);
+        r.anticausal(A, x[seg - 1 - j]);
+    }
+    // (2) states across the lanes
+    s.template scan<true>(A, seg);
+    r.template scan<false>(A, seg);
+    // (3) the outputs: the causal part, then the anticausal part added
+    const float2 zero = f2(0.f, 0.f);
+#pragma unroll 4
+    for (int j = 0; j < seg; ++j) {
+        s.causal(A, x[j]);
+        o0[j] = s.weigh(A, s.s0, 1.f, zero);
+        if constexpr (MOM) o1[j] = s.weigh(A, s.s1, -1.f, zero);
+    }
+#pragma unroll 4
+    for (int j = seg - 1; j >= 0; --j) {
+        o0[j] = r.weigh(A, r.s0, 1.f, o0[j]);
+        if constexpr (MOM) o1[j] = r.weigh(A, r.s1, 1.f, o1[j]);
+        r.anticausal(A, x[j]);
+    }
+}
+
+// Place of sample i of a line pair in its shared-memory layout, for i advancing by 32.
+struct LineAt {
+    int seg, str, q, r, dq, dr;
+    __device__ __forceinline__ LineAt(int i, int seg_)
+        : seg(seg_), str(seg_ | 1), q(i / seg_), r(i % seg_), dq(32 / seg_), dr(32 % seg_) {}
+    __device__ __forceinline__ int at() const { return q * str + r; }
+    __device__ __forceinline__ void next() {
+        q += dq;
+        r += dr;
+        if (r >= seg) { r -= seg; ++q; }
+    }
+};
+
+// Shared float2's of a pair of lines of n samples with `arrays` arrays; 4 more than a multiple of 32,
+// so that the 4 column pairs x 8 rows a warp stages at a time spread over the banks.
+__host__ __device__ constexpr int rec_pair_floats2(int n, int arrays) { return arrays * 32 * (((n + 31) / 32) | 1) + 4; }
+
+template <bool MOM>
+__global__ void __launch_bounds__(32 * kRecPairs) rec_rows_scan(const __grid_constant__ RecursiveLaunch L, int nblk) {
+    const ImageDesc& D = L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x / nblk)];
+    const int H = D.H, W = D.W, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int u = (blockIdx.x % nblk) * kRecLines + 2 * wid;
+    if (!rec_scans(H, W) || u >= H) return;   // no block-wide barrier below
+    const int seg = (W + 31) / 32, str = seg | 1;
+    const bool two = u + 1 < H;
+    const RecAxis ax(MOM ? D.rc : D.rc_self, 1);
+    extern __shared__ __align__(16) float2 rsm2[];
+    float2* x = rsm2 + wid * rec_pair_floats2(W, MOM ? 3 : 2);
+    float2 *o0 = x + 32 * str, *o1 = MOM ? o0 + 32 * str : o0;
+    {
+        LineAt p(lane, seg);
+        const size_t second = two ? (size_t)D.pitch : 0;   // one row: filtered twice, written once
+        // one loop per type, its 32 loads unconditional and in flight together (a type test or a
+        // bounds branch between them would put one memory round trip after another)
+        auto stage = [&](auto* row) {
+            for (int t = 0; t < seg; t += 16) {
+                float2 h[16];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const int v = min(32 * (t + q) + lane, W - 1);
+                    h[q] = f2((float)__ldg(row + v), (float)__ldg(row + second + v));
+                }
+#pragma unroll
+                for (int q = 0; q < 16; ++q)
+                    if (t + q < seg) {
+                        x[p.at()] = 32 * (t + q) + lane < W ? h[q] : f2(0.f, 0.f);
+                        p.next();
+                    }
+            }
+        };
+        if (D.dtype == ITC_U8) stage(reinterpret_cast<const unsigned char*>(D.data) + (size_t)u * D.pitch);
+        else stage(reinterpret_cast<const float*>(D.data) + (size_t)u * D.pitch);
+    }
+    __syncwarp();
+    filter_lines<MOM>(ax, x, o0, o1, seg, str);
+    __syncwarp();
+    float* P0 = L.fields + (MOM ? D.field_off + 3 * D.plane_floats : D.self_off + D.plane_floats) + (size_t)u * D.fpitch;
+    float* P1 = P0 + D.plane_floats;   // T_v (moments only)
+    const int fp = D.fpitch;
+    LineAt p(lane, seg);
+#pragma unroll 4
+    for (int t = 0; t < seg; ++t, p.next()) {
+        const int v = 32 * t + lane;
+        if (v < W) {
+            const float2 a = o0[p.at()];
+            P0[v] = a.x;
+            if (two) P0[fp + v] = a.y;
+            if constexpr (MOM) {
+                const float2 m = o1[p.at()];
+                P1[v] = m.x;
+                if (two) P1[fp + v] = m.y;
+            }
+        }
+    }
+}
+
+// PART 0: A and F_u from T; 1: F_v from T_v; 2: A_s (self-overlap pass).  0 and 2 with the S_XX share.
+template <int PART>
+__global__ void __launch_bounds__(32 * kRecPairs) rec_cols_scan(const __grid_constant__ RecursiveLaunch L, int nblk) {
+    constexpr bool MOM = PART == 0;
+    const ImageDesc& D = L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x / nblk)];
+    const int H = D.H, W = D.W, fp = D.fpitch, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int blk = blockIdx.x % nblk, v0 = blk * kRecLines;
+    if (!rec_scans(H, W) || v0 >= W) return;
+    const int seg = (H + 31) / 32, str = seg | 1, ls = rec_pair_floats2(H, MOM ? 3 : 2);
+    extern __shared__ __align__(16) float2 rsm2[];
+    __shared__ double red[kRecPairs];
+    const long long pl = D.plane_floats;
+    const float* T = L.fields + (PART == 2 ? D.self_off + pl : D.field_off + (3 + PART) * pl);
+    float* A = L.fields + (PART == 2 ? D.self_off : D.field_off + 2 * PART * pl);
+    // when the CTA moves columns between global and shared memory: this thread's column pair and
+    // first row (a warp moves 8 row pieces of 32 bytes)
+    const int c = tid & (kRecPairs - 1), r0 = tid / kRecPairs, v = v0 + 2 * c;
+    static_assert(32 * kRecPairs / kRecPairs == 32, "LineAt advances by 32 rows");
+    const bool in = v < W, in2 = v + 1 < W;
+    float2* const xc = rsm2 + c * ls;                // the arrays of this thread's column pair
+    float2* const xw = rsm2 + wid * ls;              // and of this warp's
+    {
+        LineAt p(r0, seg);
+        for (int t = 0; t < seg; ++t, p.next()) {   // copies of 8 bytes, zeros outside the image
+            const int u = 32 * t + r0;
+            const bool ok = in && u < H;
+            const float* src = ok ? T + (size_t)u * fp + v : T;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(xc + p.at());
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
+        }
+    }
+    // h of 16 rows at a time for the S_XX share, the first of them loaded while the columns arrive
+    float2 hv[PART != 1 ? 16 : 1];
+    auto load_h = [&](int tb) {   // unconditional loads, as in rec_rows_scan
+        const size_t pitch = (size_t)D.pitch;
+        const int va = min(v, W - 1), vb = min(v + 1, W - 1);
+        auto take = [&](auto* h) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const size_t o = (size_t)min(32 * (tb + q) + r0, H - 1) * pitch;
+                hv[q] = f2((float)__ldg(h + o + va), (float)__ldg(h + o + vb));
+            }
+        };
+        // byte pairs on 2-byte boundaries with one load each (an odd W leaves a padding byte in the
+        // last pair, weighed with 0 below): a warp's load touches 8 image rows whatever it takes from each
+        const unsigned char* hb = reinterpret_cast<const unsigned char*>(D.data);
+        if (D.dtype == ITC_U8 && ((pitch | reinterpret_cast<size_t>(hb)) & 1) == 0) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const size_t o = (size_t)min(32 * (tb + q) + r0, H - 1) * pitch;
+                const uchar2 b = __ldg(reinterpret_cast<const uchar2*>(hb + o + (va & ~1)));
+                hv[q] = f2((float)b.x, (float)b.y);
+            }
+        } else if (D.dtype == ITC_U8) {
+            take(hb);
+        } else {
+            take(reinterpret_cast<const float*>(D.data));
+        }
+    };
+    if constexpr (PART != 1) load_h(0);
+    const RecAxis ax(PART == 2 ? D.rc_self : D.rc, 0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (v0 + 2 * wid < W) filter_lines<MOM>(ax, xw, xw + 32 * str, xw + (MOM ? 64 : 32) * str, seg, str);
+    __syncthreads();
+    double hs = 0.0;
+    LineAt p(r0, seg);
+    for (int tb = 0; tb < seg; tb += 16) {
+        if constexpr (PART != 1)
+            if (tb > 0) load_h(tb);
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int u = 32 * (tb + q) + r0;
+            if (tb + q < seg) {
+                if (in && u < H) {
+                    // a pair's second column past the image lies in the row padding
+                    const size_t o = (size_t)u * fp + v;
+                    float2 a = xc[32 * str + p.at()];
+                    if (!in2) a.y = 0.f;
+                    *reinterpret_cast<float2*>(A + o) = a;
+                    if constexpr (MOM) {
+                        float2 m = xc[64 * str + p.at()];
+                        if (!in2) m.y = 0.f;
+                        *reinterpret_cast<float2*>(A + pl + o) = m;
+                    }
+                    if constexpr (PART != 1) sum = fmaf(hv[q].x, a.x, fmaf(hv[q].y, a.y, sum));
+                }
+                p.next();
+            }
+            if constexpr (PART != 1)
+                if (q % 4 == 3) {
+                    hs += (double)sum;
+                    sum = 0.f;
+                }
+        }
+    }
+    if constexpr (PART != 1) {
+        for (int o = 16; o > 0; o >>= 1) hs += __shfl_xor_sync(0xffffffffu, hs, o);
+        if (lane == 0) red[wid] = hs;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int q = 0; q < kRecPairs; ++q) t += red[q];
+            L.partials[(PART == 0 ? D.partial_off : D.sxx_off) + blk] = t;
+        }
+    }
+}
+
 // Along v: a warp takes 32 rows, one lane per row, and walks them in 32 x 32 tiles staged in
 // shared memory (rows of 33 floats), so every global load and store is a coalesced row segment
 // while each lane runs its row's recursion on the staged tile.
@@ -48,6 +389,7 @@ template <bool MOM>   // MOM: the moment fields too (else the self-overlap pass:
 __global__ void __launch_bounds__(32 * kRecRowWarps) rec_rows_kernel(const __grid_constant__ RecursiveLaunch L) {
     const ImageDesc& D = rec_image(L);
     const int H = D.H, W = D.W, fp = D.fpitch, pitch = D.pitch;
+    if (rec_scans(H, W)) return;
     float* P0 = L.fields + (MOM ? D.field_off + 3 * D.plane_floats : D.self_off + D.plane_floats);
     float* P1 = P0 + D.plane_floats;   // T_v (moments only)
     const RecCoef& rc = MOM ? D.rc : D.rc_self;
@@ -162,6 +504,7 @@ template <bool MOM>
 __global__ void __launch_bounds__(kRecColThreads) rec_cols_kernel(const __grid_constant__ RecursiveLaunch L) {
     const ImageDesc& D = rec_image(L);
     const int H = D.H, W = D.W, fp = D.fpitch;
+    if (rec_scans(H, W)) return;
     const long long pl = D.plane_floats;
     const float* T = L.fields + (MOM ? D.field_off + 3 * pl : D.self_off + pl);
     const float* Tv = T + pl;
@@ -268,10 +611,34 @@ __global__ void __launch_bounds__(kRecColThreads) rec_cols_kernel(const __grid_c
 
 }  // namespace
 
+static cudaError_t launch_scan(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s) {
+    max_H = max_H < kRecMaxLine ? max_H : kRecMaxLine;
+    max_W = max_W < kRecMaxLine ? max_W : kRecMaxLine;
+    auto go = [&](auto k, int nlines, int len, int arrays) -> cudaError_t {
+        const size_t smem = (size_t)kRecPairs * rec_pair_floats2(len, arrays) * sizeof(float2);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const int nblk = (nlines + kRecLines - 1) / kRecLines;
+        k<<<(unsigned)(nimg * nblk), 32 * kRecPairs, smem, s>>>(L, nblk);
+        return cudaGetLastError();
+    };
+    cudaError_t e;
+    if (L.mode == 0) {
+        if ((e = go(rec_rows_scan<true>, max_H, max_W, 3)) != cudaSuccess) return e;
+        if ((e = go(rec_cols_scan<0>, max_W, max_H, 3)) != cudaSuccess) return e;
+        return go(rec_cols_scan<1>, max_W, max_H, 2);
+    }
+    if ((e = go(rec_rows_scan<false>, max_H, max_W, 2)) != cudaSuccess) return e;
+    return go(rec_cols_scan<2>, max_W, max_H, 2);
+}
+
 cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s) {
     if (nimg <= 0 || max_H <= 0 || max_W <= 0) return cudaSuccess;
+    cudaError_t e = launch_scan(L, nimg, max_H, max_W, s);
+    if (e != cudaSuccess || rec_scans(max_H, max_W)) return e;
+    // images with a longer side
     const size_t smem = (size_t)kRecRowWarps * kRecTileFloats * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(rec_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(rec_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(rec_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
