@@ -210,7 +210,7 @@ struct BackwardLaunch {
     const int* img_status;      // per-image status words of the fields pass, or nullptr
 };
 
-constexpr int kChamferMaxW = 1024;   // chamfer rows: 32 lanes x 4 columns x 8 chunks
+constexpr int kChamferMaxW = 1024;   // chamfer rows: 32 lanes x 32 columns
 
 struct RecursiveLaunch {
     const ImageDesc* descs;
@@ -224,7 +224,7 @@ struct RecursiveLaunch {
 struct ChamferLaunch {
     const ImageDesc* descs;
     float* out;                 // padded per-pixel layout (pad_off, rows of fpitch floats)
-    const int* order;           // image of each warp (B ints, most pixels first)
+    const int* order;           // image of each CTA (B ints, most pixels first)
     int B;
 };
 
