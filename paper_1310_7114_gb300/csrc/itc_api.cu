@@ -199,7 +199,7 @@ size_t plan_layout(int B, size_t* desc_off, size_t* ints_off, size_t* tmap_off =
     // per class an image list and a tile prefix (an image is in at most two classes: its
     // fields class and its self-overlap class), then the backward image order
     const size_t n = align_up((size_t)((5 + kGroupInts) * (size_t)B + kMaxClasses + 2) * sizeof(int), 256);
-    const size_t m = align_up((size_t)B * sizeof(CUtensorMap), 256);
+    const size_t m = align_up((size_t)2 * B * sizeof(CUtensorMap), 256);   // fields pass, self-overlap pass
     if (desc_off) *desc_off = h;
     if (ints_off) *ints_off = h + d;
     if (tmap_off) *tmap_off = h + d + n;
@@ -253,9 +253,10 @@ int relayout(PlanHeader* h, ImageDesc* descs, int* ints, CUtensorMap* tmaps) {
         ClassInfo& ci = h->cls[c];
         if (ci.tma && !ci.use_plain)
             for (int i = 0; i < ci.nimg && ci.tma; ++i) {
-                const ImageDesc& d = descs[ints[ci.list_off + i]];
+                const int b = ints[ci.list_off + i];
+                const ImageDesc& d = descs[b];
                 if (!encode_input_map(d.data, d.H, d.W, d.pitch, d.dtype, ci.taps.R[0], ci.tile_h,
-                                      tmaps + ints[ci.list_off + i]))
+                                      tmaps + (ci.self ? h->B + b : b)))
                     ci.tma = 0;
             }
         // the plain-load kernel has one tile height per lattice dimension
@@ -304,8 +305,9 @@ cudaError_t launch_fields_any(FieldsLaunch& L, bool tma, int begin, int end, int
                               cudaStream_t s) {
     L.tile_base = begin;
     if (end <= begin) return cudaSuccess;
-    if (tma && fields_tma_supported(ndim, Ru, Rv)) return launch_fields_tma(L, end, Ru, dtype, s);
+    if (tma && fields_tma_supported(ndim, dtype, Ru, Rv, L.absolute != 0)) return launch_fields_tma(L, end, Ru, dtype, s);
     if (ndim == 3) return launch_fields3d(L, end, Ru, Rv, s);
+    if (fields_stg_supported(ndim, dtype, Ru, Rv, L.absolute != 0)) return launch_fields_stg(L, end, Ru, dtype, s);
     return launch_fields(L, end - begin, Ru, Rv, ndim, dtype, s);
 }
 
@@ -427,7 +429,7 @@ int itc_fields(const itc_image* img, const itc_params* p, float* fields, double*
     const long long nt = tiles_of(L.one);
     if (nt > 0x7fffffffLL) return ITC_ERR_UNSUPPORTED;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const bool tma = fields_tma_supported(img->ndim, L.taps.R[0], L.taps.R[1]) &&
+    const bool tma = fields_tma_supported(img->ndim, img->dtype, L.taps.R[0], L.taps.R[1], L.absolute != 0) &&
                      encode_input_map(img, L.taps.R[0], &L.tmap_one);
     // status ITC_OK unless a wait gives up; no tiles handed out yet
     rc = cuda_status(cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s));
@@ -435,12 +437,16 @@ int itc_fields(const itc_image* img, const itc_params* p, float* fields, double*
     rc = cuda_status(launch_fields_any(L, tma, 0, (int)nt, L.taps.R[0], L.taps.R[1], img->ndim, img->dtype, s));
     if (rc) return rc;
     if (sxx && has_self_pass(p, img->ndim)) {
-        // V(X) at its own width: the same tiles again (plain staging), S_XX partials only
+        // V(X) at its own width: the same tiles again, S_XX partials only
         make_taps(p, img->ndim, &L.taps, true);
         L.mode = 2;
         L.absolute = 0;
         L.test_stall = 0;
-        rc = cuda_status(launch_fields_any(L, false, 0, (int)nt, L.taps.R[0], L.taps.R[1], img->ndim, img->dtype, s));
+        const bool tma2 = fields_tma_supported(img->ndim, img->dtype, L.taps.R[0], L.taps.R[1], false) &&
+                          encode_input_map(img, L.taps.R[0], &L.tmap_one);
+        rc = cuda_status(cudaMemsetAsync(L.counter, 0, sizeof(int), s));
+        if (rc) return rc;
+        rc = cuda_status(launch_fields_any(L, tma2, 0, (int)nt, L.taps.R[0], L.taps.R[1], img->ndim, img->dtype, s));
         if (rc) return rc;
     }
     if (sxx) rc = cuda_status(launch_reduce_sxx(L.partials, (int)nt, sxx, s));
@@ -526,7 +532,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         ci.self = self ? 1 : 0;
         ci.tile_h = tile_h_of(nd);
         ci.recursive = rec;
-        ci.tma = !self && !rec && fields_tma_supported(ci.ndim, ci.taps.R[0], ci.taps.R[1]) ? 1 : 0;
+        ci.tma = !rec && fields_tma_supported(ci.ndim, ci.dtype, ci.taps.R[0], ci.taps.R[1], false) ? 1 : 0;
         return c;
     };
     for (int b = 0; b < B; ++b) {
@@ -600,7 +606,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
     {
         // the largest count over "every class at its smallest tile height" bounds any tuning
         for (int c = 0; c < h->ncls; ++c)
-            if (h->cls[c].tma) h->cls[c].tile_h = 32;
+            if (h->cls[c].tma && !h->cls[c].self && fields_tma_heights(h->cls[c].taps.R[0])) h->cls[c].tile_h = 32;
         int rc = relayout(h, descs, ints, tmaps);
         if (rc) return rc;
         pcap = h->total_tiles;
@@ -726,11 +732,11 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
         L.partials = v.partials;
         L.tile_h = ci.tile_h;
         L.absolute = 0;
-        L.tmaps = reinterpret_cast<const CUtensorMap*>(pd + h->tmap_off);
+        L.tmaps = reinterpret_cast<const CUtensorMap*>(pd + h->tmap_off) + (ci.self ? h->B : 0);
         L.grid_per_sm = ci.grid_per_sm;
         L.mode = ci.self ? 1 : 0;
         L.status = v.status;
-        L.test_stall = stall;
+        L.test_stall = ci.self ? 0 : stall;
         // this launch's tile counter (unique per class and first image, so that range calls on
         // other streams do not share it), zeroed first
         L.counter = v.counters + ci.list_off + p0;
@@ -746,7 +752,7 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
             R.mode = L.mode;
             rc = cuda_status(launch_recursive(R, p1 - p0, h->max_dim[0], h->max_dim[1], s));
         } else {
-            rc = cuda_status(launch_fields_any(L, ci.tma != 0 && !ci.use_plain && !ci.self, t0, t1, ci.taps.R[0],
+            rc = cuda_status(launch_fields_any(L, ci.tma != 0 && !ci.use_plain, t0, t1, ci.taps.R[0],
                                                ci.taps.R[1], ci.ndim, ci.dtype, s));
         }
         if (rc) return rc;
@@ -822,9 +828,11 @@ int itc_autotune(void* plan_host, void* plan_dev, void* ws, size_t ws_bytes, int
         if (ci.tma) {
             cands[nc++] = {0, 64, 0};
             cands[nc++] = {0, 64, 1};
-            cands[nc++] = {0, 32, 0};
-            cands[nc++] = {0, 32, 1};
-            cands[nc++] = {0, 128, 0};
+            if (fields_tma_heights(ci.taps.R[0])) {
+                cands[nc++] = {0, 32, 0};
+                cands[nc++] = {0, 32, 1};
+                cands[nc++] = {0, 128, 0};
+            }
         }
         cands[nc++] = {1, 64, 0};
         float best = 3.4e38f;
@@ -875,6 +883,7 @@ int itc_plan_configure(void* plan_host, void* plan_dev, int c, int tile_h, int g
     if (staging == 1 && !ci.tma) return ITC_ERR_UNSUPPORTED;
     if (staging == 1 ? (tile_h != 32 && tile_h != 64 && tile_h != 128) : tile_h != tile_h_of(ci.ndim))
         return ITC_ERR_INVALID_ARG;
+    if (staging == 1 && tile_h != 64 && !fields_tma_heights(ci.taps.R[0])) return ITC_ERR_UNSUPPORTED;
     ci.use_plain = staging ? 0 : 1;
     ci.tile_h = tile_h;
     ci.grid_per_sm = grid_per_sm;

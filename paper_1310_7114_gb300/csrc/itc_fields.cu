@@ -1,6 +1,7 @@
 // itc_fields.cu -- truncated separable Gaussian fields of 2-D lattice images (Sec. 3.1, Sec. 5)
-// with plain staging (rows that are not on 16-byte boundaries, radii without a compiled TMA
-// kernel); gray images as [u, v, g] lattices are in itc_fields3d.cu.
+// with plain staging, for what the tiled kernel (itc_fields_tma.cuh) is not compiled for: other or
+// unequal radii, and absolute moments on rows that are not on 16-byte boundaries; gray images as
+// [u, v, g] lattices are in itc_fields3d.cu.
 //
 // One CTA computes a TH x 64 tile of output sites:
 //   1. the input tile plus an R-wide halo is staged in shared memory as float (zero outside the
@@ -10,9 +11,9 @@
 //   3. pass along u over the staged rows: A = g_u * T, F_u = (d g_u) * T or g_u * (u T),
 //      F_v = g_u * T_v, written with 128-bit stores;
 //   4. epilogue: the tile's share of S_XX = sum_x h(x) A(x) (V(X) of Eq. (1)) as one double.
-// Tiles whose staged input is all zero only write zeros.  For the radii the parameter sets use
-// (6, 9, 12) both passes are fully unrolled with the taps in the constant bank; other radii
-// run the same passes with runtime loops.
+// Tiles whose staged input is all zero only write zeros.  For absolute moments at radii 6, 9 and 12 both
+// passes are fully unrolled with the taps in the constant bank; the rest runs the same passes with
+// runtime loops.
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -314,7 +315,7 @@ cudaError_t launch_one(const FieldsLaunch& L, int nblocks, int Ru, int Rv, cudaS
 
 template <bool ABS, int DTYPE, int TH>
 cudaError_t dispatch_radius(const FieldsLaunch& L, int nblocks, int Ru, int Rv, cudaStream_t s) {
-    if (Ru == Rv) {
+    if constexpr (ABS) if (Ru == Rv) {   // centred moments at these radii go through the tiled kernel
         if (Ru == 6) return launch_one<6, 6, ABS, DTYPE, TH>(L, nblocks, Ru, Rv, s);
         if (Ru == 9) return launch_one<9, 9, ABS, DTYPE, TH>(L, nblocks, Ru, Rv, s);
         if (Ru == 12) return launch_one<12, 12, ABS, DTYPE, TH>(L, nblocks, Ru, Rv, s);

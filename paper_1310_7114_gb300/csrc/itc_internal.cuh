@@ -132,7 +132,8 @@ struct PlanHeader {
     int run_nlarge[2], run_ngroups[2];   // iteration groups: the 2-D images of more than kRunThreads
                                 // vectors (one per group), the other 2-D groups, then the same in 3-D
     double run_work[2];         // most (iters + 1) M^2 of the former, per dimension
-    long long tmap_off;         // bytes from plan start to CUtensorMap[B] (input tiles)
+    long long tmap_off;         // bytes from plan start to CUtensorMap[2 B]: input tiles of the fields
+                                // pass, then of the self-overlap pass
     long long pad_floats;       // sum H*fpitch (padded per-pixel layout)
     int has_recursive;          // some class computes its fields by recursion
     ClassInfo cls[kMaxClasses];
@@ -168,6 +169,7 @@ struct FieldsLaunch {
     int mode;                   // 0: every field plane; 1: A only, into the A_s plane, S_XX
                                 // partials at sxx_off (self-overlap pass); 2: S_XX partials only
     int* counter;               // tensor-tile path: chunks of tiles handed out so far (0 at launch)
+    int chunk;                  // tensor-tile path, set at launch: tiles per chunk
     int* status;                // device status words: one per image of the plan (batched) or one
                                 // for the call (single image); a CTA whose bounded wait gives up
                                 // writes ITC_ERR_TIMEOUT for every image it still owned tiles of
@@ -251,9 +253,21 @@ cudaError_t launch_reduce_sxx(const double* partials, int n, double* out, cudaSt
 cudaError_t launch_fields3d(const FieldsLaunch& L, int ntiles, int R_u, int R_v, cudaStream_t s);
 // TMA-staged 2-D fields (itc_fields_tma.cu): the radii it is compiled for, its box per radius
 // and data type, and its launch.
-bool fields_tma_supported(int ndim, int Ru, int Rv);
+bool fields_tma_supported(int ndim, int dtype, int Ru, int Rv, bool absolute);
+bool fields_tma_heights(int R);   // compiled for 32- and 128-row tiles too
 int fields_tma_box(int dtype, int R, int tile_h, int* box_w, int* box_h);
 cudaError_t launch_fields_tma(const FieldsLaunch& L, int ntiles, int R, int dtype, cudaStream_t s);
+// The same tiles with the input copied by the threads: rows on any boundary, 64-row tiles, centred moments.
+bool fields_stg_supported(int ndim, int dtype, int Ru, int Rv, bool absolute);
+cudaError_t launch_fields_stg(const FieldsLaunch& L, int ntiles, int R, int dtype, cudaStream_t s);
+cudaError_t launch_fields_stg_u8(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_stg_f32(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_stg_self_u8(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_stg_self_f32(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_tma_u8(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_tma_f32(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_tma_self_u8(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
+cudaError_t launch_fields_tma_self_f32(const FieldsLaunch& L, int ntiles, int R, cudaStream_t s);
 // The iterations (itc_run.cu) of one lattice dimension: nlarge images of more than kRunThreads
 // codebook vectors and the others.  With L.groups: large_ctas groups of the former, then ctas groups
 // of the others; else both are the range's image count.  work: most (iters + 1) M^2 of a large image.
