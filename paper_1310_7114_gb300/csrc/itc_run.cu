@@ -23,6 +23,8 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -52,8 +54,11 @@ __device__ __forceinline__ float lattice_round(float x, int n) {
 
 // Position of the padding entries past an image's last vector: its weight 2^(-1e38 c) is 0
 constexpr float kFar = 1e19f;
-// Pair-loop steps whose arithmetic is kept in flight together
-constexpr int kPairU = 4;
+// Pair-loop steps whose arithmetic is kept in flight together: kPairU, and half of them for the rest;
+// positions are padded to the latter.  (4096 ragged shapes, 50 iterations: 0.426 ms with 8, 0.438
+// with 4, 0.470 with 2; one image of M = 128, 100 iterations: 171, 186 and 225 us.)
+constexpr int kPairU = 8;
+constexpr int kPairPad = kPairU;   // two positions per step
 
 struct Sums {
     float sxw, sww;
@@ -139,7 +144,7 @@ __device__ __forceinline__ float2 pair_weights(const float4 q, const float2 z, c
     return f2(ex2_ftz(x.x), ex2_ftz(x.y));
 }
 
-// Pair sums of one vector over mp positions (a multiple of 2 kPairU): (x_j, x_j+1, y_j, y_j+1) per
+// Pair sums of one vector over mp positions (a multiple of kPairPad): (x_j, x_j+1, y_j, y_j+1) per
 // even j with one 16-byte broadcast load, z by itself; the even j accumulate in the .x halves and
 // the odd j in the .y halves.  kPairU steps run side by side: a lone image has one warp per SM
 // sub-partition, and one step at a time it waited for its chain of load, exponent and ex2 (74
@@ -150,22 +155,27 @@ __device__ __forceinline__ void pair_sums(const float* sxy, const float* sz, int
     float2 nw[ND], sp = f2(0.f, 0.f), ep[ND];
 #pragma unroll
     for (int i = 0; i < ND; ++i) { nw[i] = f2(-w[i], -w[i]); ep[i] = f2(0.f, 0.f); }
-#pragma unroll 1
-    for (int j = 0; j < mp; j += 2 * kPairU) {
-        float2 g[kPairU], d[kPairU][ND];
+    int j = 0;
+    auto block = [&](auto steps) {
+        constexpr int U = decltype(steps)::value;
+        float2 g[U], d[U][ND];
 #pragma unroll
-        for (int u = 0; u < kPairU; ++u) {
+        for (int u = 0; u < U; ++u) {
             const float4 q = *reinterpret_cast<const float4*>(sxy + 2 * (j + 2 * u));
             const float2 z = ND == 3 ? *reinterpret_cast<const float2*>(sz + j + 2 * u) : f2(0.f, 0.f);
             g[u] = pair_weights<ND, ISO>(q, z, nw, nc, d[u]);
         }
 #pragma unroll
-        for (int u = 0; u < kPairU; ++u) {
+        for (int u = 0; u < U; ++u) {
             sp = __fadd2_rn(sp, g[u]);
 #pragma unroll
             for (int i = 0; i < ND; ++i) ep[i] = __ffma2_rn(g[u], d[u][i], ep[i]);
         }
-    }
+        j += 2 * U;
+    };
+#pragma unroll 1
+    while (j + 2 * kPairU <= mp) block(std::integral_constant<int, kPairU>());
+    if (j < mp) block(std::integral_constant<int, kPairU / 2>());
     s = sp.x + sp.y;
 #pragma unroll
     for (int i = 0; i < ND; ++i) E[i] = ep[i].x + ep[i].y;
@@ -173,7 +183,7 @@ __device__ __forceinline__ void pair_sums(const float* sxy, const float* sz, int
 
 // Positions split by the parity of j, for threads that sum the even or the odd j alone: four j are
 // stored as (x_j, x_j+2, y_j, y_j+2) and (x_j+1, x_j+3, y_j+1, y_j+3).
-constexpr int kHalfPad = 4 * kPairU;   // positions are padded to whole pair-loop blocks of one parity
+constexpr int kHalfPad = 2 * kPairU;   // positions are padded to whole (half) blocks of one parity
 __device__ __forceinline__ int half_at(int k) { return (k >> 2) * 8 + (k & 1) * 4 + ((k >> 1) & 1); }
 __device__ __forceinline__ int half_atz(int k) { return (k >> 2) * 4 + (k & 1) * 2 + ((k >> 1) & 1); }
 
@@ -188,17 +198,18 @@ __device__ __forceinline__ void half_sums(const float* pos, const float* posz, i
     s = 0.f;
     pos += 4 * half;
     posz += 2 * half;
-#pragma unroll 1
-    for (int j = 0; j < mp; j += kHalfPad) {
-        float2 g[kPairU], d[kPairU][ND];
+    int j = 0;
+    auto block = [&](auto steps) {
+        constexpr int U = decltype(steps)::value;
+        float2 g[U], d[U][ND];
 #pragma unroll
-        for (int u = 0; u < kPairU; ++u) {
+        for (int u = 0; u < U; ++u) {
             const float4 q = *reinterpret_cast<const float4*>(pos + 2 * j + 8 * u);
             const float2 z = ND == 3 ? *reinterpret_cast<const float2*>(posz + j + 4 * u) : f2(0.f, 0.f);
             g[u] = pair_weights<ND, ISO>(q, z, nw, nc, d[u]);
         }
 #pragma unroll
-        for (int u = 0; u < kPairU; ++u) {
+        for (int u = 0; u < U; ++u) {
             s += g[u].x;
             s += g[u].y;
 #pragma unroll
@@ -207,7 +218,11 @@ __device__ __forceinline__ void half_sums(const float* pos, const float* posz, i
                 E[i] = fmaf(g[u].y, d[u][i].y, E[i]);
             }
         }
-    }
+        j += 4 * U;
+    };
+#pragma unroll 1
+    while (j + 4 * kPairU <= mp) block(std::integral_constant<int, kPairU>());
+    if (j < mp) block(std::integral_constant<int, kPairU / 2>());
 }
 
 // n / a, correctly rounded, with the correctly rounded reciprocal ra of a at hand (Markstein, IBM
@@ -301,7 +316,7 @@ __device__ __forceinline__ void iterate_group(const RunLaunch& L, const int* grp
     if (!has) D.M = 0;
     const PairWidths<ND> pw(Dg);
     const bool mine = kl < D.M;
-    const int mp = (D.M + 2 * kPairU - 1) / (2 * kPairU) * (2 * kPairU);
+    const int mp = (D.M + kPairPad - 1) / kPairPad * kPairPad;
     float* sxy = s_pos + sub * SPAN * ND;
     float* sz = sxy + 2 * SPAN;
     auto sync_image = [&]() {
@@ -627,7 +642,7 @@ __device__ __forceinline__ void iterate_large(const RunLaunch& L) {
     const Img D = load_img(L, Dg);
     const PairWidths<ND> pw(Dg);
     const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    constexpr int PAD = SPLIT ? kHalfPad : 2 * kPairU;
+    constexpr int PAD = SPLIT ? kHalfPad : kPairPad;
     const int mp = (M + PAD - 1) / PAD * PAD;
     const int share = large_share(M, csize), k0 = min(M, rank * share), own = min(M, k0 + share) - k0;
     extern __shared__ __align__(16) float lsm[];
