@@ -582,6 +582,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         h->max_dim[1] = d.W > h->max_dim[1] ? d.W : h->max_dim[1];
         h->max_dim[2] = d.G > h->max_dim[2] ? d.G : h->max_dim[2];
         h->ndim_mask |= 1 << d.ndim;
+        h->kind_mask |= 1 << (d.ndim == 3 ? kSegGray : (d.dtype == ITC_U8 ? kSegBytes : kSegWeights));
     }
     h->fields_floats = foff;
     h->total_pixels = ghoff;
@@ -974,8 +975,10 @@ int itc_segment(const void* plan_host, const void* plan_dev, const float* W, sho
     L.descs = reinterpret_cast<const ImageDesc*>(pd + h->desc_off);
     L.W = W;
     L.labels = labels;
+    L.split = 1;
     L.order = reinterpret_cast<const int*>(pd + h->ints_off) + h->bwd_order_off;
-    return cuda_status(launch_segment(L, h->B, h->max_M, reinterpret_cast<cudaStream_t>(stream)));
+    return cuda_status(launch_segment(L, h->B, h->max_M, h->max_bwd_tiles, h->kind_mask,
+                                      reinterpret_cast<cudaStream_t>(stream)));
 }
 
 int itc_plan_classes(const void* plan_host) {

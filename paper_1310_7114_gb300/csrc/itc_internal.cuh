@@ -111,6 +111,7 @@ struct PlanHeader {
     int max_M;
     int max_dim[3];             // largest H, W, G over the plan's images
     int ndim_mask;              // bit 2: the plan has 2-D images; bit 3: it has 3-D images
+    int kind_mask;              // bit kSegBytes / kSegWeights / kSegGray: it has such images
     long long total_pixels;     // sum H*W (grad_h layout)
     long long fields_floats;    // sum of every image's field planes
     long long total_tiles;
@@ -230,11 +231,14 @@ struct ChamferLaunch {
     int B;
 };
 
+constexpr int kSegBytes = 0, kSegWeights = 1, kSegGray = 2;   // 2-D bytes, 2-D weights, 3-D
+
 struct SegmentLaunch {
     const ImageDesc* descs;
     const float* W;
     short* labels;              // per image H x W at gh_off
     const int* order;           // image of each CTA (B ints, most pixels first)
+    int split;                  // CTAs per image (set at launch)
 };
 
 constexpr int kBwdTileH = 64;   // backward pixel tile: 64 rows x 64 columns
@@ -275,7 +279,8 @@ cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas,
                        int ndim);
 cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
 cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
-cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, cudaStream_t s);
+// max_blocks: most 64 x 64 pixel blocks of one image; kinds: bit kSeg* for each kind of image in the plan
+cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int kinds, cudaStream_t s);
 cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long pixel_tiles, int max_image_tiles,
                             cudaStream_t s);
 }  // namespace itc
