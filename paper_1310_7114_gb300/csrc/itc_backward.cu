@@ -6,9 +6,10 @@
 // (tau = sigma: the data kernel and its fields; rho: the codebook pair kernel; A_s: the field of h
 // at the width s of V(X); rho = s = tau unless set apart, and then A_s = A.)
 //
-// Kernel 1 (one CTA per image): window sums a_k, D_k around round(w_k) read directly from the
-// image (kernel evaluated at the real w_k, one warp per k), the M x M sums s_k, E_k (one warp
-// per k, xor-shuffle reduction), S_XW, S_WW, grad_W and two per-image scalars for kernel 2.
+// Kernel 1 (one CTA per image): a_k, D_k from the stored fields or, for a real-valued codebook, as
+// window sums around round(w_k) read directly from the image (kernel evaluated at the real w_k, one
+// warp per k), the M x M sums s_k, E_k (one thread per k), S_XW, S_WW, grad_W and two per-image
+// scalars for kernel 2.
 // Kernel 2 (one CTA per image, over its 64 x 64 pixel tiles): the codebooks whose box meets a
 // tile are listed in k order (ballot compaction), their Gaussians are stamped onto the tile in
 // that order -- the transposed form of the gather in the forward update -- and every pixel
@@ -16,6 +17,7 @@
 #include <math.h>
 
 #include "itc_internal.cuh"
+#include "itc_pairs.cuh"
 
 namespace itc {
 namespace {
@@ -28,45 +30,96 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-// 2^x by the PTX instruction ex2.approx.ftz.f32 (relative error about 2^-22; results below the
-// smallest normal float flush to zero)
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ int lattice_round_i(float x, int n) {
     float r = floorf(x + 0.5f);
     return (int)fminf(fmaxf(r, 0.f), (float)(n - 1));
-}
-__device__ __forceinline__ float pixel_weight(const ImageDesc& D, int u, int v) {
-    const size_t o = (size_t)u * D.pitch + v;
-    if (D.ndim == 3) return D.weight ? __ldg(D.weight + o) : 1.f;
-    if (D.dtype == ITC_U8) return (float)__ldg(reinterpret_cast<const unsigned char*>(D.data) + o);
-    return __ldg(reinterpret_cast<const float*>(D.data) + o);
 }
 __device__ __forceinline__ int pixel_gray(const ImageDesc& D, int u, int v) {
     return (int)__ldg(reinterpret_cast<const unsigned char*>(D.data) + (size_t)u * D.pitch + v);
 }
 
-__global__ void __launch_bounds__(kRunThreads) bwd_codebook_kernel(const __grid_constant__ BackwardLaunch L) {
-    const int img = L.img_base + blockIdx.x;
-    const ImageDesc& D = L.descs[img];
-    const int M = D.M, nd = D.ndim, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int nw = blockDim.x >> 5;
+// Dynamic shared floats of the codebook kernel: positions, z, then a (1), D (3), s (1), E (3) per vector
+__host__ __device__ constexpr size_t codebook_smem_floats(int M) { return (size_t)((M + kPairPad - 1) / kPairPad * kPairPad) * 11; }
+
+__device__ __forceinline__ float tree8(const float (&x)[8]) {
+    return ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+}
+
+// a_k and D_k summed over the box around round(w_k) with the kernel at the real w_k, by the calling warp: a
+// lane per column of the box (in turns of 32), the loads of eight rows in flight together.  (8 weight
+// images of 256 x 256, M = 32, R = 9: 41 us with the positions dealt out one by one, a division and a
+// dependent load each, to four warps per image; 13 us now, with sixteen.)
+template <int ND>
+__device__ __forceinline__ void window_sums(const ImageDesc& D, float w0, float w1, float w2, float* sa, float* sD) {
+    const int lane = threadIdx.x & 31;
+    const int H = D.H, Wd = D.W, Ru = D.R[0], Rv = D.R[1], Rg = D.R[2];
+    const float c0 = D.inv2s2[0], c1 = D.inv2s2[1], c2 = D.inv2s2[2];
+    const int r0 = lattice_round_i(w0, H), r1 = lattice_round_i(w1, Wd), r2 = ND == 3 ? lattice_round_i(w2, D.G) : 0;
+    const int ua = max(0, r0 - Ru), ub = min(H - 1, r0 + Ru), va = max(0, r1 - Rv), vb = min(Wd - 1, r1 + Rv);
+    float a = 0.f, d0 = 0.f, d1 = 0.f, d2 = 0.f;
+    for (int vt = va; vt <= vb; vt += 32) {
+        const int v = vt + lane, vc = min(v, vb);
+        const float dv = (float)v - w1, ev = dv * dv * c1;
+        auto rows = [&](auto* h) {   // h: weights (null: ones); unconditional loads from clamped places
+            for (int u = ua; u <= ub; u += 8) {
+                float x[8], y[8], gl[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const size_t o = (size_t)min(u + q, ub) * D.pitch + vc;
+                    x[q] = h ? (float)__ldg(h + o) : 1.f;
+                    gl[q] = ND == 3 ? (float)__ldg(reinterpret_cast<const unsigned char*>(D.data) + o) : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float du = (float)(u + q) - w0, dg = gl[q] - w2;
+                    float e = du * du * c0 + ev;
+                    if (ND == 3) e += dg * dg * c2;
+                    const bool in = u + q <= ub && v <= vb && x[q] != 0.f && (ND == 2 || fabsf(gl[q] - (float)r2) <= (float)Rg);
+                    x[q] = in ? x[q] * expf(-e) : 0.f;
+                    y[q] = x[q] * du;
+                    gl[q] = ND == 3 ? x[q] * dg : 0.f;
+                }
+                const float g = tree8(x);   // pairwise: a lane adds up to 2 R + 1 rows
+                a += g;
+                d0 += tree8(y);
+                d1 = fmaf(g, dv, d1);
+                if (ND == 3) d2 += tree8(gl);
+            }
+        };
+        if (ND == 3) rows(D.weight);
+        else if (D.dtype == ITC_U8) rows(reinterpret_cast<const unsigned char*>(D.data));
+        else rows(reinterpret_cast<const float*>(D.data));
+    }
+    a = warp_sum_f(a);
+    d0 = warp_sum_f(d0);
+    d1 = warp_sum_f(d1);
+    d2 = warp_sum_f(d2);
+    if (lane == 0) {
+        sa[0] = a;
+        sD[0] = d0;
+        sD[1] = d1;
+        sD[2] = d2;
+    }
+}
+
+template <int ND>
+__device__ __forceinline__ void codebook_image(const BackwardLaunch& L, const ImageDesc& D, int img) {
+    const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nw = blockDim.x >> 5, mp = (M + kPairPad - 1) / kPairPad * kPairPad;
     extern __shared__ __align__(16) float sm[];
-    float* sw = sm;
-    float* sa = sw + 3 * M;
-    float* sD = sa + M;
-    float* ss = sD + 3 * M;
-    float* sE = ss + M;
-    __shared__ double red[4];
+    float* sxy = sm;             // positions in pairs (pair_sums), padded
+    float* sz = sxy + 2 * mp;
+    float* sa = sz + mp;
+    float* sD = sa + mp;         // 3 per vector
+    float* ss = sD + 3 * mp;
+    float* sE = ss + mp;
+    __shared__ double red[4], coef[6];
+    __shared__ double s_px[32];
 
     // S_XX from the image's tile partials: warp 0 alone, or for a gray image (a partial per
-    // slice tile) every warp a strided share with eight loads in flight per lane, the warp sums
-    // added in warp order
-    __shared__ double s_px[32];
-    const int nws = nd == 3 ? nw : 1;
+    // slice tile) the first four warps a strided share each with eight loads in flight per lane, the
+    // warp sums added in warp order
+    const int nws = ND == 3 ? kRunThreads / 32 : 1;
     if (wid < nws) {
         const long long nt = D.sxx_tiles, step = 32LL * nws;
         double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -79,93 +132,52 @@ __global__ void __launch_bounds__(kRunThreads) bwd_codebook_kernel(const __grid_
         if (lane == 0) s_px[wid] = t;
     }
     const float* Wk = L.W + D.w_off;
-    for (int k = tid; k < M; k += blockDim.x)
-        for (int i = 0; i < 3; ++i) sw[k * 3 + i] = i < nd ? Wk[k * nd + i] : 0.f;
-    __syncthreads();
-    double sxx = 0;
-    for (int q = 0; q < nws; ++q) sxx += s_px[q];
-    const float c0 = D.inv2s2[0], c1 = D.inv2s2[1], c2 = D.inv2s2[2];
-    const int Ru = D.R[0], Rv = D.R[1], Rg = D.R[2];
-
+    const int n[3] = {D.H, D.W, D.G};
+    int off_lattice = 0;
+    for (int k = tid; k < mp; k += blockDim.x) {
+        float w[3] = {kFar, kFar, kFar};
+        if (k < M) {
+#pragma unroll
+            for (int i = 0; i < ND; ++i) {
+                w[i] = Wk[k * ND + i];
+                off_lattice |= (w[i] != rintf(w[i])) || !(w[i] >= 0.f) || !(w[i] <= (float)(n[i] - 1));
+            }
+        }
+        sxy[(k >> 1) * 4 + (k & 1)] = w[0];
+        sxy[(k >> 1) * 4 + 2 + (k & 1)] = w[1];
+        sz[k] = w[2];
+    }
     // a_k and D_k: on the lattice (every w_k integral and inside it) they are the stored field
     // values at w_k; otherwise window sums around round(w_k) with the kernel at the real w_k
-    int off_lattice = 0;
-    for (int k = tid; k < M; k += blockDim.x)
-        for (int i = 0; i < nd; ++i) {
-            const float w = sw[k * 3 + i];
-            const int ni = i == 0 ? D.H : (i == 1 ? D.W : D.G);
-            off_lattice |= (w != rintf(w)) || !(w >= 0.f) || !(w <= (float)(ni - 1));
-        }
     const bool gather = !__syncthreads_or(off_lattice);
-    if (gather) {
-        const float* A = L.fields + D.field_off;
-        for (int k = tid; k < M; k += blockDim.x) {
-            const int r0 = (int)sw[k * 3], r1 = (int)sw[k * 3 + 1], r2 = nd == 3 ? (int)sw[k * 3 + 2] : 0;
-            const long long o = ((long long)r2 * D.H + r0) * D.fpitch + r1;
-            sa[k] = __ldg(A + o);
-            for (int i = 0; i < 3; ++i) sD[k * 3 + i] = i < nd ? __ldg(A + (i + 1) * D.plane_floats + o) : 0.f;
+    auto at = [&](int k, int i) { return i == 2 ? sz[k] : sxy[(k >> 1) * 4 + 2 * i + (k & 1)]; };
+    if (!gather)
+        for (int k = wid; k < M; k += nw) window_sums<ND>(D, at(k, 0), at(k, 1), at(k, 2), sa + k, sD + 3 * k);
+    // codebook interaction sums: one thread per k, the gathers in flight beside them
+    const PairWidths<ND> pw(D);
+    const float* A = L.fields + D.field_off;
+    for (int k = tid; k < M; k += blockDim.x) {
+        float w[ND], E[ND], s, a = 0.f, f[ND];
+#pragma unroll
+        for (int i = 0; i < ND; ++i) w[i] = at(k, i);
+        if (gather) {
+            const long long o = ((long long)(ND == 3 ? (int)w[ND - 1] : 0) * D.H + (int)w[0]) * D.fpitch + (int)w[1];
+            a = __ldg(A + o);
+#pragma unroll
+            for (int i = 0; i < ND; ++i) f[i] = __ldg(A + (i + 1) * D.plane_floats + o);
         }
-    } else {
-        for (int k = wid; k < M; k += nw) {
-            const float w0 = sw[k * 3], w1 = sw[k * 3 + 1], w2 = sw[k * 3 + 2];
-            const int r0 = lattice_round_i(w0, D.H), r1 = lattice_round_i(w1, D.W);
-            const int r2 = nd == 3 ? lattice_round_i(w2, D.G) : 0;
-            const int ua = max(0, r0 - Ru), ub = min(D.H - 1, r0 + Ru);
-            const int va = max(0, r1 - Rv), vb = min(D.W - 1, r1 + Rv);
-            const int nv = vb - va + 1, npos = (ub - ua + 1) * nv;
-            float a = 0.f, d0 = 0.f, d1 = 0.f, d2 = 0.f;
-            for (int p = lane; p < npos; p += 32) {
-                const int u = ua + p / nv, v = va + p % nv;
-                const float h = pixel_weight(D, u, v);
-                if (h == 0.f) continue;
-                const float du = (float)u - w0, dv = (float)v - w1;
-                float dg = 0.f;
-                if (nd == 3) {
-                    const int gl = pixel_gray(D, u, v);
-                    if (abs(gl - r2) > Rg) continue;
-                    dg = (float)gl - w2;
-                }
-                const float g = h * expf(-(du * du * c0 + dv * dv * c1 + dg * dg * c2));
-                a += g;
-                d0 = fmaf(g, du, d0);
-                d1 = fmaf(g, dv, d1);
-                d2 = fmaf(g, dg, d2);
-            }
-            a = warp_sum_f(a);
-            d0 = warp_sum_f(d0);
-            d1 = warp_sum_f(d1);
-            d2 = warp_sum_f(d2);
-            if (lane == 0) {
-                sa[k] = a;
-                sD[k * 3] = d0;
-                sD[k * 3 + 1] = d1;
-                sD[k * 3 + 2] = d2;
-            }
-        }
-    }
-    // codebook interaction sums: one thread per k, every j in order
-    {
-        const float q0 = (float)(1.4426950408889634 * (double)D.pinv2s2[0]);
-        const float q1 = (float)(1.4426950408889634 * (double)D.pinv2s2[1]);
-        const float q2 = (float)(1.4426950408889634 * (double)D.pinv2s2[2]);
-        for (int k = tid; k < M; k += blockDim.x) {
-            const float wk0 = sw[k * 3], wk1 = sw[k * 3 + 1], wk2 = sw[k * 3 + 2];
-            float s_ = 0.f, e0 = 0.f, e1 = 0.f, e2 = 0.f;
-            for (int j = 0; j < M; ++j) {
-                const float d0 = sw[j * 3] - wk0, d1 = sw[j * 3 + 1] - wk1, d2 = sw[j * 3 + 2] - wk2;
-                const float g = exp2f(-(d0 * d0 * q0 + d1 * d1 * q1 + d2 * d2 * q2));
-                s_ += g;
-                e0 = fmaf(g, d0, e0);
-                e1 = fmaf(g, d1, e1);
-                e2 = fmaf(g, d2, e2);
-            }
-            ss[k] = s_;
-            sE[k * 3] = e0;
-            sE[k * 3 + 1] = e1;
-            sE[k * 3 + 2] = e2;
+        if (ND == 2 && pw.iso) pair_sums<ND, ND == 2>(sxy, sz, mp, w, pw.nc, s, E);
+        else pair_sums<ND, false>(sxy, sz, mp, w, pw.nc, s, E);
+        ss[k] = s;
+        if (gather) sa[k] = a;
+#pragma unroll
+        for (int i = 0; i < ND; ++i) {
+            sE[k * 3 + i] = E[i];
+            if (gather) sD[k * 3 + i] = f[i];
         }
     }
     __syncthreads();
+    const double gD = L.grad_dcs ? (double)L.grad_dcs[img] : 1.0;
     if (wid == 0) {
         double x = 0, y = 0;
         int e = 0;
@@ -176,46 +188,58 @@ __global__ void __launch_bounds__(kRunThreads) bwd_codebook_kernel(const __grid_
         }
         x = warp_sum_d(x);
         y = warp_sum_d(y);
-        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        e = __reduce_add_sync(0xffffffffu, e);
+        // on a lane each: the coefficients of E and D in grad_W per axis, and of the two terms of grad_h
+        double sxx = 0;
+        for (int q = 0; q < nws; ++q) sxx += s_px[q];   // written before the barriers above
+        const int i = lane < 6 ? lane % 3 : 0;
+        const double width = lane < 3 ? (double)D.rho[i] : (double)D.sigma[i];
+        const double den = lane < 3 ? width * width * y : (lane < 6 ? width * width * x : (lane == 6 ? sxx : x));
+        const double c = 2.0 * gD / den;
+        if (lane < 6) coef[lane] = c;
+        if (lane == 6) L.scal[img * 4 + 0] = c;
+        if (lane == 7) L.scal[img * 4 + 1] = c;
         if (lane == 0) {
             red[0] = x;
             red[1] = y;
             red[2] = (double)e;
+            red[3] = sxx;
         }
     }
     __syncthreads();
-    const double sxw = red[0], sww = red[1];
-    const double gD = L.grad_dcs ? (double)L.grad_dcs[img] : 1.0;
     if (L.grad_W) {
         float* gW = L.grad_W + D.w_off;
         for (int k = tid; k < M; k += blockDim.x)
-            for (int i = 0; i < nd; ++i) {
-                const double t2 = (double)D.sigma[i] * (double)D.sigma[i];
-                const double r2 = (double)D.rho[i] * (double)D.rho[i];
-                gW[k * nd + i] = (float)(gD * 2.0 * ((double)sE[k * 3 + i] / (r2 * sww) -
-                                                     (double)sD[k * 3 + i] / (t2 * sxw)));
-            }
+#pragma unroll
+            for (int i = 0; i < ND; ++i)
+                gW[k * ND + i] = (float)(coef[i] * (double)sE[k * 3 + i] - coef[3 + i] * (double)sD[k * 3 + i]);
     }
-    if (tid == 0) {
-        L.scal[img * 4 + 0] = 2.0 * gD / sxx;
-        L.scal[img * 4 + 1] = 2.0 * gD / sxw;
-        if (L.stats) {
-            itc_stats r;
-            r.sxw = sxw;
-            r.sww = sww;
-            r.sxx = sxx;
-            r.c = sxw / sww;
-            r.dcs = sxw > 0 ? log(sww) + log(sxx) - 2.0 * log(sxw) + D.dcs_const : INFINITY;
-            r.empty = (int)red[2];
-            r.moved = 0;
-            r.iters_done = 0;
-            const int dev_status = L.img_status ? L.img_status[img] : ITC_OK;
-            r.status = dev_status == ITC_ERR_TIMEOUT ? ITC_ERR_TIMEOUT
-                       : (!(sxw > 0) || !isfinite(r.dcs) ? ITC_ERR_NONFINITE
-                          : (r.empty > 0 ? ITC_WARN_EMPTY_SUPPORT : ITC_OK));
-            L.stats[img] = r;
-        }
+    if (tid == 0 && L.stats) {
+        const double sxw = red[0], sww = red[1], sxx = red[3];
+        itc_stats r;
+        r.sxw = sxw;
+        r.sww = sww;
+        r.sxx = sxx;
+        r.c = sxw / sww;
+        r.dcs = sxw > 0 ? log(sww) + log(sxx) - 2.0 * log(sxw) + D.dcs_const : INFINITY;
+        r.empty = (int)red[2];
+        r.moved = 0;
+        r.iters_done = 0;
+        const int dev_status = L.img_status ? L.img_status[img] : ITC_OK;
+        r.status = dev_status == ITC_ERR_TIMEOUT ? ITC_ERR_TIMEOUT
+                   : (!(sxw > 0) || !isfinite(r.dcs) ? ITC_ERR_NONFINITE
+                      : (r.empty > 0 ? ITC_WARN_EMPTY_SUPPORT : ITC_OK));
+        L.stats[img] = r;
     }
+}
+
+constexpr int kCodebookThreads = 512;   // most threads of a codebook CTA
+
+__global__ void __launch_bounds__(kCodebookThreads, 1) bwd_codebook_kernel(const __grid_constant__ BackwardLaunch L) {
+    const int img = L.img_base + blockIdx.x;
+    const ImageDesc& D = L.descs[img];
+    if (D.ndim == 3) codebook_image<3>(L, D, img);
+    else codebook_image<2>(L, D, img);
 }
 
 constexpr int kChunk = 64;   // codebooks staged per round in the pixel kernel
@@ -464,10 +488,11 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
 cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long pixel_tiles, int max_image_tiles,
                             cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
-    const size_t smem1 = (size_t)max_M * kCodebookSmemFloats * sizeof(float);
+    const size_t smem1 = codebook_smem_floats(max_M) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(bwd_codebook_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
     if (e != cudaSuccess) return e;
-    bwd_codebook_kernel<<<B, kRunThreads, smem1, s>>>(L);
+    // few images: as many threads as keep a CTA's window sums and pair sums short
+    bwd_codebook_kernel<<<B, B <= kSoloImages ? kCodebookThreads : kRunThreads, smem1, s>>>(L);
     e = cudaGetLastError();
     if (e != cudaSuccess || !L.grad_h || pixel_tiles <= 0) return e;
     const size_t smem2 = (size_t)max_M * (16 + 7 * sizeof(int));   // list records, positions, sites, tile list

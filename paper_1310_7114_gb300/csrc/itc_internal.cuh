@@ -21,10 +21,6 @@ constexpr int kSoloImages = 152;    // up to one image per SM of the GPU: iterat
 // kRunThreads / 16 image indices.  Images with M <= span share one CTA, span threads each.
 constexpr int kGroupMax = 8;
 constexpr int kGroupInts = 2 + kGroupMax;
-// Dynamic shared floats per codebook vector of the backward-codebook kernel: w (3), a (1), D (3),
-// s (1), E (3).
-constexpr int kCodebookSmemFloats = 11;
-
 // Truncated, unnormalised 1-D Gaussian taps of one parameter class, computed on the host in
 // double and rounded once to float:  g[d + R] = exp(-d^2 / (2 sigma^2)),  dg[d + R] = d g[d + R].
 struct Taps {
