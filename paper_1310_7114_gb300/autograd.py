@@ -42,7 +42,7 @@ def _forward(ctx, sigma, trunc, budget: Optional[int], tensors):
         itc.run_budget(plan, W, ctx.ws, st)
     ctx.plan, ctx.W = plan, W
     ctx.shapes = [tuple(w.shape) for w in Ws]
-    return st.view(torch.float64).view(B, 7)[:, 0].float()
+    return st.view(torch.float64)[::7].float()   # the first of each record's seven
 
 
 def _backward(ctx, grad):
@@ -53,8 +53,9 @@ def _backward(ctx, grad):
         itc.backward(plan, W, grad_dcs=grad.float().contiguous(), grad_W=gW, grad_h=gh)
     else:
         itc.backward_budget(plan, W, ctx.ws, grad_dcs=grad.float().contiguous(), grad_W=gW, grad_h=gh)
-    ghs = [gh[plan.gh_offsets[b]:plan.gh_offsets[b + 1]].view(plan.shapes[b]) for b in range(plan.B)]
-    gWs = [gW[plan.w_offsets[b]:plan.w_offsets[b + 1]].view(ctx.shapes[b]) for b in range(plan.B)]
+    gh_off, w_off = plan.gh_offsets.tolist(), plan.w_offsets.tolist()
+    ghs = [gh.as_strided(s, (s[1], 1), o) for s, o in zip(plan.shapes, gh_off)]
+    gWs = [gW.as_strided(s, (s[1], 1), o) for s, o in zip(ctx.shapes, w_off)]
     return ghs, gWs
 
 

@@ -80,10 +80,11 @@ int check_params(const itc_params* p, int ndim) {
 
 // g[d + R] = exp(-d^2 / (2 sigma^2)) and d g[d + R], computed in double, rounded once.
 void fill_taps(float sigma, int R, float* g, float* dg) {
-    for (int d = -R; d <= R; ++d) {
+    for (int d = 0; d <= R; ++d) {
         const double v = exp(-((double)d * d) / (2.0 * (double)sigma * sigma));
-        g[d + R] = (float)v;
-        dg[d + R] = (float)(d * v);
+        g[R + d] = g[R - d] = (float)v;
+        dg[R + d] = (float)(d * v);
+        dg[R - d] = (float)(-d * v);
     }
 }
 
@@ -120,7 +121,12 @@ void make_taps(const itc_params* p, int ndim, Taps* t, bool self = false) {
     }
     if (rec) return;   // no masks
     fill_taps(t->sigma[0], t->R[0], t->gu, t->dgu);
-    fill_taps(t->sigma[1], t->R[1], t->gv, t->dgv);
+    if (t->sigma[1] == t->sigma[0]) {
+        memcpy(t->gv, t->gu, sizeof(t->gu));
+        memcpy(t->dgv, t->dgu, sizeof(t->dgu));
+    } else {
+        fill_taps(t->sigma[1], t->R[1], t->gv, t->dgv);
+    }
     if (ndim == 3) fill_taps(t->sigma[2], t->R[2], t->gg, t->dgg);
     float a = 0.f, b = 0.f;
     for (int d = 0; d <= 2 * t->R[1]; ++d) {
@@ -247,7 +253,8 @@ bool encode_input_map(const itc_image* img, int R, CUtensorMap* out) {
 }
 
 // Tile grid, class tile prefixes and S_XX partial offsets of a plan from each class's tile
-// height; per-image tensor maps follow the tile height.  The int area keeps its size.
+// height; per-image tensor maps follow the tile height (tmaps null: counting tiles only).  The int area
+// keeps its size.
 int relayout(PlanHeader* h, ImageDesc* descs, int* ints, CUtensorMap* tmaps) {
     for (int c = 0; c < h->ncls; ++c) {
         ClassInfo& ci = h->cls[c];
@@ -255,8 +262,8 @@ int relayout(PlanHeader* h, ImageDesc* descs, int* ints, CUtensorMap* tmaps) {
             for (int i = 0; i < ci.nimg && ci.tma; ++i) {
                 const int b = ints[ci.list_off + i];
                 const ImageDesc& d = descs[b];
-                if (!encode_input_map(d.data, d.H, d.W, d.pitch, d.dtype, ci.taps.R[0], ci.tile_h,
-                                      tmaps + (ci.self ? h->B + b : b)))
+                if (tmaps && !encode_input_map(d.data, d.H, d.W, d.pitch, d.dtype, ci.taps.R[0], ci.tile_h,
+                                               tmaps + (ci.self ? h->B + b : b)))
                     ci.tma = 0;
             }
         // the plain-load kernel has one tile height per lattice dimension
@@ -431,8 +438,8 @@ int itc_fields(const itc_image* img, const itc_params* p, float* fields, double*
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const bool tma = fields_tma_supported(img->ndim, img->dtype, L.taps.R[0], L.taps.R[1], L.absolute != 0) &&
                      encode_input_map(img, L.taps.R[0], &L.tmap_one);
-    // status ITC_OK unless a wait gives up; no tiles handed out yet
-    rc = cuda_status(cudaMemsetAsync(L.status, 0, 2 * sizeof(int), s));
+    // status ITC_OK unless a wait gives up; no tiles handed out yet (a counter for each of the two passes)
+    rc = cuda_status(cudaMemsetAsync(L.status, 0, 3 * sizeof(int), s));
     if (rc) return rc;
     rc = cuda_status(launch_fields_any(L, tma, 0, (int)nt, L.taps.R[0], L.taps.R[1], img->ndim, img->dtype, s));
     if (rc) return rc;
@@ -444,8 +451,7 @@ int itc_fields(const itc_image* img, const itc_params* p, float* fields, double*
         L.test_stall = 0;
         const bool tma2 = fields_tma_supported(img->ndim, img->dtype, L.taps.R[0], L.taps.R[1], false) &&
                           encode_input_map(img, L.taps.R[0], &L.tmap_one);
-        rc = cuda_status(cudaMemsetAsync(L.counter, 0, sizeof(int), s));
-        if (rc) return rc;
+        L.counter = L.status + 2;
         rc = cuda_status(launch_fields_any(L, tma2, 0, (int)nt, L.taps.R[0], L.taps.R[1], img->ndim, img->dtype, s));
         if (rc) return rc;
     }
@@ -608,7 +614,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         // the largest count over "every class at its smallest tile height" bounds any tuning
         for (int c = 0; c < h->ncls; ++c)
             if (h->cls[c].tma && !h->cls[c].self && fields_tma_heights(h->cls[c].taps.R[0])) h->cls[c].tile_h = 32;
-        int rc = relayout(h, descs, ints, tmaps);
+        int rc = relayout(h, descs, ints, nullptr);
         if (rc) return rc;
         pcap = h->total_tiles;
         for (int c = 0; c < h->ncls; ++c) h->cls[c].tile_h = tile_h_of(h->cls[c].ndim);
@@ -711,9 +717,15 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
     const int* ints = reinterpret_cast<const int*>(pd + h->ints_off);
     const ImageDesc* hdescs = reinterpret_cast<const ImageDesc*>(reinterpret_cast<const unsigned char*>(plan_host) +
                                                                  h->desc_off);
-    // the images' status words start at ITC_OK; a fields CTA whose bounded wait gives up sets them
-    if (b1 > b0 && cudaMemsetAsync(v.status + b0, 0, (size_t)(b1 - b0) * sizeof(int), s) != cudaSuccess)
-        return ITC_ERR_CUDA;
+    // the images' status words start at ITC_OK (a fields CTA whose bounded wait gives up sets them) and the
+    // launches' tile counters at zero; a call for the whole batch clears both with one memset
+    const bool whole = b0 == 0 && b1 == h->B;
+    int last_list = 0;
+    for (int c = 0; c < h->ncls; ++c) last_list = std::max(last_list, h->cls[c].list_off);
+    const size_t clear = whole ? (size_t)(reinterpret_cast<unsigned char*>(v.counters + last_list + 1) -
+                                          reinterpret_cast<unsigned char*>(v.status))
+                               : (size_t)(b1 - b0) * sizeof(int);
+    if (b1 > b0 && cudaMemsetAsync(v.status + b0, 0, clear, s) != cudaSuccess) return ITC_ERR_CUDA;
     for (int c = 0; c < h->ncls; ++c) {
         const ClassInfo& ci = h->cls[c];
         const int p0 = lower_pos(hints + ci.list_off, ci.nimg, b0), p1 = lower_pos(hints + ci.list_off, ci.nimg, b1);
@@ -741,7 +753,7 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
         // this launch's tile counter (unique per class and first image, so that range calls on
         // other streams do not share it), zeroed first
         L.counter = v.counters + ci.list_off + p0;
-        if (cudaMemsetAsync(L.counter, 0, sizeof(int), s) != cudaSuccess) return ITC_ERR_CUDA;
+        if (!whole && cudaMemsetAsync(L.counter, 0, sizeof(int), s) != cudaSuccess) return ITC_ERR_CUDA;
         int rc;
         if (ci.recursive) {
             RecursiveLaunch R;

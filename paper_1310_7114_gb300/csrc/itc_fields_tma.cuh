@@ -867,12 +867,11 @@ cudaError_t launch_tma(const FieldsLaunch& L, int ntiles, cudaStream_t s) {
     auto k = fields_tma_kernel<R, ABS, DTYPE, TH, AO, STG, LM>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, smem)) != cudaSuccess) return e;
+    static ResidentCtas resident;
+    int sms = 0, per_sm = 0;
+    if ((e = resident.get(k, kThreads, smem, &sms, &per_sm)) != cudaSuccess) return e;
     if (L.grid_per_sm > 0 && L.grid_per_sm < per_sm) per_sm = L.grid_per_sm;   // tuned persistent grid
-    const int cap = sms * (per_sm > 0 ? per_sm : 1);
+    const int cap = sms * per_sm;
     const int n = ntiles - L.tile_base;
     // one 1024 x 1024 image is 256 tiles: 64 CTAs with four each left most SMs idle (27 -> 16 us at R =
     // 12); 100 ragged shapes, 5.5 tiles per CTA, still gain from single tiles (byte images at R = 9: 58 ->

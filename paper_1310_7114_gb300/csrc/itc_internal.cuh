@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "itc.h"
 
 namespace itc {
@@ -137,6 +139,31 @@ struct PlanHeader {
 };
 
 constexpr uint32_t kPlanMagic = 0x49544350u;  // "ITCP"
+
+// CTAs of one kernel and shared-memory size that fit on the current device at once, looked up once per
+// device (the query takes longer than a launch).  A static one per kernel.
+struct ResidentCtas {
+    static constexpr int kDevices = 64;
+    std::atomic<int> of_device[kDevices] = {};
+    template <typename K>
+    cudaError_t get(K kernel, int threads, size_t smem, int* sms, int* per_sm) {
+        int dev = 0, n = 0, p = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const int known = dev < kDevices ? of_device[dev].load(std::memory_order_relaxed) : 0;
+        if (known) {   // SM count and CTAs per SM, packed
+            *sms = known >> 8;
+            *per_sm = known & 255;
+            return cudaSuccess;
+        }
+        if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kernel, threads, smem)) != cudaSuccess) return e;
+        *sms = n;
+        *per_sm = p > 0 ? p : 1;
+        if (dev < kDevices) of_device[dev].store((n << 8) | (*per_sm & 255), std::memory_order_relaxed);
+        return cudaSuccess;
+    }
+};
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from itertools import accumulate
 from typing import Optional, Sequence
 
 import numpy as np
@@ -181,9 +182,11 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    # the current stream's handle without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _width3(x, fill):
@@ -329,19 +332,18 @@ class Plan:
         _check(lib().itc_plan(B, imgs, Ms, ps, stride, ctypes.cast(self.host, _P), nbytes, ctypes.byref(ws)),
                "itc_plan")
         dev = device if device is not None else images[0].device
-        blob = np.frombuffer(self.host.raw, dtype=np.uint8)
-        self.dev = torch.from_numpy(blob.copy()).to(dev)
+        self.dev = torch.frombuffer(self.host, dtype=torch.uint8).to(dev, copy=True)
         self.ws_bytes = int(ws.value)
         # the whole batch's fields; a plan used only through the budgeted calls needs none of it
         self.ws = torch.empty(max(self.ws_bytes, 256), dtype=torch.uint8, device=dev) if allocate_ws else None
-        self.pixels = int(lib().itc_plan_pixels(ctypes.cast(self.host, _P)))
-        self.w_offsets = np.concatenate([[0], np.cumsum([m * d for m, d in zip(self.M, ndims)])]).astype(np.int64)
-        self.gh_offsets = np.concatenate([[0], np.cumsum([h * w for h, w in self.shapes])]).astype(np.int64)
+        self.pixels = int(lib().itc_plan_pixels(self.host_ptr))
+        self.w_offsets = np.array([0, *accumulate(m * d for m, d in zip(self.M, ndims))], np.int64)
+        self.gh_offsets = np.array([0, *accumulate(h * w for h, w in self.shapes)], np.int64)
         self._keep = (images, weights)
 
     @property
-    def host_ptr(self):
-        return ctypes.cast(self.host, _P)
+    def host_ptr(self) -> int:
+        return ctypes.addressof(self.host)
 
     def budget_bytes(self, budget_bytes: int = 0) -> int:
         """itc_plan_budget_bytes: workspace of the budgeted calls within ``budget_bytes`` in all
