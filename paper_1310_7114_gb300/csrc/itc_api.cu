@@ -1197,22 +1197,23 @@ static int backward_images(const PlanHeader* h, const void* plan_host, const voi
     L.img_status = v.status;
     if (whole) {
         L.bwd_order = reinterpret_cast<const int*>(pd + h->ints_off) + h->bwd_order_off;
-        return cuda_status(launch_backward(L, h->B, h->max_M, h->bwd_tiles, h->max_bwd_tiles, s));
+        return cuda_status(launch_backward(L, h->B, h->max_M, h->bwd_tiles, h->max_bwd_tiles, h->ndim_mask, s));
     }
     // an image range: its CTAs in image order
     const ImageDesc* hd = reinterpret_cast<const ImageDesc*>(reinterpret_cast<const unsigned char*>(plan_host) +
                                                              h->desc_off);
     long long tiles = 0;
-    int max_tiles = 0, max_M = 0;
+    int max_tiles = 0, max_M = 0, ndim_mask = 0;
     for (int b = b0; b < b1; ++b) {
         const int t = hd[b].bwd_tiles_u * hd[b].bwd_tiles_v;
         tiles += t;
         max_tiles = std::max(max_tiles, t);
         max_M = std::max(max_M, hd[b].M);
+        ndim_mask |= 1 << hd[b].ndim;
     }
     L.bwd_order = nullptr;
     L.img_base = b0;
-    return cuda_status(launch_backward(L, b1 - b0, max_M, tiles, max_tiles, s));
+    return cuda_status(launch_backward(L, b1 - b0, max_M, tiles, max_tiles, ndim_mask, s));
 }
 
 int itc_backward(const void* plan_host, const void* plan_dev, const float* W, const float* grad_dcs,

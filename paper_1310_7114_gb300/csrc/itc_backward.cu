@@ -10,11 +10,13 @@
 // window sums around round(w_k) read directly from the image (kernel evaluated at the real w_k, one
 // warp per k), the M x M sums s_k, E_k (one thread per k), S_XW, S_WW, grad_W and two per-image
 // scalars for kernel 2.
-// Kernel 2 (one CTA per image, over its 64 x 64 pixel tiles): the codebooks whose box meets a
-// tile are listed in k order (ballot compaction), their Gaussians are stamped onto the tile in
+// Kernel 2 (per dimension; 16 x 64 pixel tiles of a warp in 2-D, 64 x 64 of a CTA in 3-D): the codebooks
+// whose box meets a tile are taken in k order (ballots), their Gaussians are stamped onto the tile in
 // that order -- the transposed form of the gather in the forward update -- and every pixel
 // combines the stored field A with the stamp.
 #include <math.h>
+
+#include <algorithm>
 
 #include "itc_internal.cuh"
 #include "itc_pairs.cuh"
@@ -245,24 +247,156 @@ __global__ void __launch_bounds__(kCodebookThreads, 1) bwd_codebook_kernel(const
     else codebook_image<2>(L, D, img);
 }
 
-constexpr int kChunk = 64;   // codebooks staged per round in the pixel kernel
+constexpr int kPixWarps = 4;    // warps of a 2-D pixel CTA
+constexpr int kPixRows = 16, kPixCols = 64;   // a warp's tile
+constexpr int kPixSlots = 16;   // codebook vectors staged per turn
+constexpr int kPixStage = kPixRows + kPixCols;   // floats of one: a, then b
 
-// Pixel pass: one CTA per image walks the image's 64 x 64 tiles (images with the most tiles
-// are launched first).  The stamp S(x) = sum_k g(x - w_k) [x in box(round(w_k))] is separable
-// in 2-D: g(x - w) = g_u(x_u - w_u) g_v(x_v - w_v) and the box is a product of two intervals,
-// so for the codebooks whose box meets a tile (listed in k order)
+// 2-D pixel pass.  The stamp S(x) = sum_k g(x - w_k) [x in box(round(w_k))] is separable:
+// g(x - w) = g_u(x_u - w_u) g_v(x_v - w_v) and the box is a product of two intervals, so for the vectors
+// whose box meets a tile, taken in k order,
 //   S(r, c) = sum_l a_l(r) b_l(c),  a_l(r) = g_u(u0 + r - w_lu) [|u0 + r - r_lu| <= R_u], ...
-// Chunks of 64 listed codebooks are staged as a (64 x 64) and b (64 x 64) in shared memory and
-// every thread accumulates a 4 x 4 block of pixels in l order (deterministic, no atomics), with
-// packed FMAs over pairs of columns.  In 3-D the g factor depends on each pixel's gray level and
-// is applied per pixel and codebook.
-__global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_constant__ BackwardLaunch L) {
+// Every warp walks 16 x 64 tiles of its image on its own: it loads the field (a lane has 8 rows x 4
+// columns), finds the vectors by ballot, stages a and b of up to 16 of them in its own shared memory and adds
+// them in l order with packed FMAs over pairs of rows (deterministic, no atomics).  HBM bounds it: 4 bytes
+// read and 4 written per pixel.  Nothing waits for other warps, so that 20 of them per SM keep loads in flight
+// (64 x 64 tiles of a CTA with a barrier per phase: 113 us for 256 images of 512 x 512, 6.3 TB/s in 85 us now;
+// 589 and 464 us for 4096 ragged images).  Row pieces of 256 bytes: fields and gradients of ragged images start
+// anywhere in a 128-byte line, and with 32 x 32 tiles the shared lines cost 514 us.
+__global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const __grid_constant__ BackwardLaunch L) {
+    // split CTAs per image: the warps take its tiles in turn
+    const int split = L.split;
+    const int img = L.bwd_order ? __ldg(L.bwd_order + blockIdx.x / split) : L.img_base + (int)(blockIdx.x / split);
+    const ImageDesc& D = L.descs[img];
+    if (D.ndim != 2) return;
+    const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int H = D.H, Wd = D.W, fpitch = D.fpitch, Ru = D.R[0], Rv = D.R[1];
+    const int tiles_v = (Wd + kPixCols - 1) / kPixCols, ntiles = tiles_v * ((H + kPixRows - 1) / kPixRows);
+    const int first = (int)(blockIdx.x % split) * kPixWarps;
+    if (first >= ntiles) return;
+    // the separable factors exp(-d^2 c) = 2^(-d^2 c log2 e), log2 e folded into the widths
+    const float l0 = (float)(1.4426950408889634 * (double)D.inv2s2[0]), l1 = (float)(1.4426950408889634 * (double)D.inv2s2[1]);
+    // the S_XX term uses the field of h at the width of V(X): A itself unless set apart
+    const float* A = L.fields + (D.self_off >= 0 ? D.self_off : D.field_off);
+    float* gh = L.grad_h + D.gh_off;
+    const float s1 = (float)L.scal[img * 4 + 0], s2 = (float)L.scal[img * 4 + 1];
+
+    extern __shared__ __align__(16) unsigned char bsm[];
+    float4* rec = reinterpret_cast<float4*>(bsm);   // per vector: position and site along u and v
+    __shared__ __align__(16) float stage[kPixWarps][kPixSlots][kPixStage];
+    const float* Wk = L.W + D.w_off;
+    for (int k = tid; k < M; k += blockDim.x) {
+        const float w0 = Wk[k * 2], w1 = Wk[k * 2 + 1];
+        rec[k] = make_float4(w0, w1, __int_as_float(lattice_round_i(w0, H)), __int_as_float(lattice_round_i(w1, Wd)));
+    }
+    __syncthreads();
+
+    static_assert(kPixSlots * kPixStage >= kPixRows * kPixCols, "a warp's stage holds a tile");
+    float(*st)[kPixStage] = stage[wid];
+    const int br = lane >> 4 << 3, bc = (lane & 15) << 2;   // a lane's 8 x 4 block of a tile
+    const bool rows16 = (Wd & 3) == 0 && (reinterpret_cast<size_t>(gh) & 15) == 0;
+    for (int t = first + wid; t < ntiles; t += split * kPixWarps) {
+        const int u0 = t / tiles_v * kPixRows, v0 = (t - t / tiles_v * tiles_v) * kPixCols;
+        const int u = u0 + lane, v = v0 + lane, nrow = min(kPixRows, H - u0);
+        // this lane's 8 x 4 block of the field, loaded first so that its latency overlaps the stamp
+        float4 f[8];
+        {
+            const float* p = A + min(v0 + bc, fpitch - 4);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f[i] = __ldg(reinterpret_cast<const float4*>(p + (size_t)min(u0 + br + i, H - 1) * fpitch));
+        }
+        float2 acc[4][4];   // row pairs, columns
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        const float fu = (float)u, fv = (float)v;
+        int ns = 0;
+        auto add = [&] {
+            __syncwarp();
+#pragma unroll 1
+            for (int l = 0; l < ns; ++l) {
+                const float4 b = *reinterpret_cast<const float4*>(&st[l][kPixRows + bc]);
+                const float4 a0 = *reinterpret_cast<const float4*>(&st[l][br]), a1 = *reinterpret_cast<const float4*>(&st[l][br + 4]);
+                const float2 a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
+                const float bj[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[i][j] = __ffma2_rn(a[i], make_float2(bj[j], bj[j]), acc[i][j]);
+            }
+            __syncwarp();
+            ns = 0;
+        };
+        for (int base = 0; base < M; base += 32) {
+            bool hit = false;
+            if (base + lane < M) {
+                const float4 r = rec[base + lane];
+                const int r0 = __float_as_int(r.z), r1 = __float_as_int(r.w);
+                hit = r0 + Ru >= u0 && r0 - Ru < u0 + kPixRows && r1 + Rv >= v0 && r1 - Rv < v0 + kPixCols;
+            }
+            unsigned bal = __ballot_sync(0xffffffffu, hit);
+            while (bal) {
+                const float4 r = rec[base + __ffs(bal) - 1];
+                bal &= bal - 1;
+                const float du = fu - r.x, dv = fv - r.y;
+                const float dv2 = (float)(v + 32) - r.y;
+                if (lane < kPixRows) st[ns][lane] = abs(u - __float_as_int(r.z)) <= Ru ? ex2_ftz(-(du * du) * l0) : 0.f;
+                st[ns][kPixRows + lane] = abs(v - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv * dv) * l1) : 0.f;
+                st[ns][kPixRows + 32 + lane] = abs(v + 32 - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv2 * dv2) * l1) : 0.f;
+                if (++ns == kPixSlots) add();
+            }
+        }
+        if (ns) add();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float* q = &acc[i >> 1][0].x + (i & 1);
+            f[i] = make_float4(s1 * f[i].x - s2 * q[0], s1 * f[i].y - s2 * q[2], s1 * f[i].z - s2 * q[4], s1 * f[i].w - s2 * q[6]);
+        }
+        if (rows16) {
+            float* out = gh + (size_t)(u0 + br) * Wd + v0 + bc;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (v0 + bc < Wd && br + i < nrow) *reinterpret_cast<float4*>(out + (size_t)i * Wd) = f[i];
+            continue;
+        }
+        // rows on any boundary: through the warp's shared memory, a row piece to each store
+        float* tile = &st[0][0];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + (br + i) * kPixCols + bc) = f[i];
+        __syncwarp();
+        float* out = gh + (size_t)u0 * Wd + v;
+        const bool in0 = v < Wd, in1 = v + 32 < Wd;
+        if (nrow == kPixRows) {
+#pragma unroll
+            for (int i = 0; i < kPixRows; ++i, out += Wd) {
+                if (in0) out[0] = tile[i * kPixCols + lane];
+                if (in1) out[32] = tile[i * kPixCols + 32 + lane];
+            }
+        } else {
+            for (int i = 0; i < nrow; ++i, out += Wd) {
+                if (in0) out[0] = tile[i * kPixCols + lane];
+                if (in1) out[32] = tile[i * kPixCols + 32 + lane];
+            }
+        }
+        __syncwarp();
+    }
+}
+
+constexpr int kChunk = 64;   // codebooks staged per round in the 3-D pixel kernel
+
+// 3-D pixel pass: one CTA per image walks the image's 64 x 64 tiles (images with the most tiles
+// are launched first).  The codebooks whose box meets a tile are listed in k order; chunks of 64 of them are
+// staged as a (64 x 64) and b (64 x 64) in shared memory and every thread accumulates a 4 x 4 block of pixels
+// in l order.  The g factor depends on each pixel's gray level and is applied per pixel and codebook.
+__global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_constant__ BackwardLaunch L) {
     // split CTAs per image (few large images): CTA s of an image takes its tiles s, s + split, ...
     const int split = L.split;
     const int img = L.bwd_order ? __ldg(L.bwd_order + blockIdx.x / split) : L.img_base + (int)(blockIdx.x / split);
     const int part = blockIdx.x % split;
     const ImageDesc& D = L.descs[img];
-    const int M = D.M, nd = D.ndim, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (D.ndim != 3) return;
+    const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int H = D.H, Wd = D.W, G = D.G, fpitch = D.fpitch, tiles_v = D.bwd_tiles_v;
     const int ntiles = D.bwd_tiles_u * D.bwd_tiles_v;
     const int Ru = D.R[0], Rv = D.R[1], Rg = D.R[2];
@@ -273,11 +407,6 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
     const float* A = L.fields + (D.self_off >= 0 ? D.self_off : D.field_off);
     float* gh = L.grad_h + D.gh_off;
     const float s1 = (float)L.scal[img * 4 + 0], s2 = (float)L.scal[img * 4 + 1];
-    // every row of this image's dD/dh starts on a 16-byte boundary (width and offset multiples of
-    // 4 floats, aligned base): the results go out as 16-byte row pieces, else through shared
-    // memory as whole row segments
-    const bool rows16 = ((Wd & 3) == 0) && ((reinterpret_cast<size_t>(gh) & 15) == 0);
-
     extern __shared__ __align__(16) unsigned char bsm[];
     // per listed codebook of the current tile one 16-byte record (position and site along u
     // and v), then the codebooks' positions, sites and the list itself
@@ -291,13 +420,13 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
 
     const float* Wk = L.W + D.w_off;
     for (int k = tid; k < M; k += blockDim.x) {
-        const float w0 = Wk[k * nd], w1 = Wk[k * nd + 1], w2 = nd == 3 ? Wk[k * nd + 2] : 0.f;
+        const float w0 = Wk[k * 3], w1 = Wk[k * 3 + 1], w2 = Wk[k * 3 + 2];
         cw[k * 3] = w0;
         cw[k * 3 + 1] = w1;
         cw[k * 3 + 2] = w2;
         cr[k * 3] = lattice_round_i(w0, H);
         cr[k * 3 + 1] = lattice_round_i(w1, Wd);
-        cr[k * 3 + 2] = nd == 3 ? lattice_round_i(w2, G) : 0;
+        cr[k * 3 + 2] = lattice_round_i(w2, G);
     }
     __syncthreads();
 
@@ -305,26 +434,15 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
     if (part >= ntiles) return;
     for (int t = part; t < ntiles; t += split) {
         const int u0 = (t / tiles_v) * kBwdTileH, v0 = (t % tiles_v) * kBwdTileW;
-        // field values of this thread's block, loaded first so their latency overlaps the stamp
-        float4 a4[4];
         int gray[4][4];
         const bool cols_in = v0 + pc < Wd;
-        if (nd == 2) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int u = min(u0 + pr + i, H - 1);
-                a4[i] = cols_in ? __ldg(reinterpret_cast<const float4*>(A + (long long)u * fpitch + v0 + pc))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int u = u0 + pr + i, v = v0 + pc + j;
+                gray[i][j] = (u < H && v < Wd) ? pixel_gray(D, u, v) : 0;
             }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int u = u0 + pr + i, v = v0 + pc + j;
-                    gray[i][j] = (u < H && v < Wd) ? pixel_gray(D, u, v) : 0;
-                }
-        }
 
         // stable compaction of the codebooks whose box meets this tile
         int nl = 0;
@@ -357,10 +475,7 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
             __syncthreads();
         }
 
-        // accumulators as column pairs (j = 0, 1 and 2, 3) of each row, the packed FMA operands
-        float2 acc2[4][2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { acc2[i][0] = make_float2(0.f, 0.f); acc2[i][1] = make_float2(0.f, 0.f); }
+        float acc[4][4] = {};
         // factor staging: each thread fills one row / column r of the factors for every fourth l
         const int sr = tid & (kBwdTileH - 1), sl = tid / kBwdTileH;
         static_assert(kBwdTileH == kBwdTileW && kThreads % kBwdTileH == 0, "square tiles, whole rows of threads");
@@ -379,89 +494,25 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
                 sb[l][sr] = bv;
             }
             __syncthreads();
-            if (nd == 2) {
-#pragma unroll 1   // unrolled, the loop spills at the 80-register budget of 3 CTAs per SM
-                for (int l = 0; l < nc; ++l) {
-                    const float4 av4 = *reinterpret_cast<const float4*>(&sa[l][pr]);
-                    const float4 bv4 = *reinterpret_cast<const float4*>(&sb[l][pc]);
-                    const float av[4] = {av4.x, av4.y, av4.z, av4.w};
-                    const float2 b01 = make_float2(bv4.x, bv4.y), b23 = make_float2(bv4.z, bv4.w);
+            for (int l = 0; l < nc; ++l) {
+                const float4 av4 = *reinterpret_cast<const float4*>(&sa[l][pr]);
+                const float4 bv4 = *reinterpret_cast<const float4*>(&sb[l][pc]);
+                const float av[4] = {av4.x, av4.y, av4.z, av4.w}, bv[4] = {bv4.x, bv4.y, bv4.z, bv4.w};
+                const int k = lk[base + l];
+                const float wg = cw[k * 3 + 2];
+                const int rg = cr[k * 3 + 2];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 ai = make_float2(av[i], av[i]);
-                        acc2[i][0] = __ffma2_rn(ai, b01, acc2[i][0]);
-                        acc2[i][1] = __ffma2_rn(ai, b23, acc2[i][1]);
-                    }
-                }
-            } else {
-                for (int l = 0; l < nc; ++l) {
-                    const float4 av4 = *reinterpret_cast<const float4*>(&sa[l][pr]);
-                    const float4 bv4 = *reinterpret_cast<const float4*>(&sb[l][pc]);
-                    const float av[4] = {av4.x, av4.y, av4.z, av4.w}, bv[4] = {bv4.x, bv4.y, bv4.z, bv4.w};
-                    const int k = lk[base + l];
-                    const float wg = cw[k * 3 + 2];
-                    const int rg = cr[k * 3 + 2];
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int gl = gray[i][j];
-                            if (abs(gl - rg) <= Rg) {
-                                const float d = (float)gl - wg;
-                                float& aij = (j & 1) ? acc2[i][j >> 1].y : acc2[i][j >> 1].x;
-                                aij = fmaf(av[i] * bv[j], expf(-d * d * c2), aij);
-                            }
+                    for (int j = 0; j < 4; ++j) {
+                        const int gl = gray[i][j];
+                        if (abs(gl - rg) <= Rg) {
+                            const float d = (float)gl - wg;
+                            acc[i][j] = fmaf(av[i] * bv[j], expf(-d * d * c2), acc[i][j]);
                         }
-                }
+                    }
             }
             __syncthreads();   // sa / sb are rewritten by the next chunk or tile
-        }
-        float acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            acc[i][0] = acc2[i][0].x; acc[i][1] = acc2[i][0].y; acc[i][2] = acc2[i][1].x; acc[i][3] = acc2[i][1].y;
-        }
-
-        if (nd == 2 && rows16) {
-            // rows of dD/dh start on 16-byte boundaries: one 16-byte store per row of the block
-            // (a warp writes two full 256-byte row segments per instruction)
-            if (cols_in) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int u = u0 + pr + i;
-                    if (u >= H) break;
-                    float* out = gh + (long long)u * Wd + v0 + pc;
-                    const float r4[4] = {s1 * a4[i].x - s2 * acc[i][0], s1 * a4[i].y - s2 * acc[i][1],
-                                         s1 * a4[i].z - s2 * acc[i][2], s1 * a4[i].w - s2 * acc[i][3]};
-                    if (v0 + pc + 3 < Wd) {
-                        *reinterpret_cast<float4*>(out) = make_float4(r4[0], r4[1], r4[2], r4[3]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (v0 + pc + j < Wd) out[j] = r4[j];
-                    }
-                }
-            }
-            continue;
-        }
-        if (nd == 2) {
-            // the thread's 4 x 4 results go through shared memory (sa is free after the last
-            // chunk's barrier), so that each warp writes 32 consecutive pixels of a row
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                *reinterpret_cast<float4*>(&sa[pr + i][pc]) =
-                    make_float4(s1 * a4[i].x - s2 * acc[i][0], s1 * a4[i].y - s2 * acc[i][1],
-                                s1 * a4[i].z - s2 * acc[i][2], s1 * a4[i].w - s2 * acc[i][3]);
-            __syncthreads();
-            const int r0 = tid >> 6, c = tid & 63;   // rows r0, r0 + 4, ..., column c
-            if (v0 + c < Wd) {
-                const int nrow = min(16, max(0, (H - u0 - r0 + 3) >> 2));
-                float* gp = gh + (long long)(u0 + r0) * Wd + v0 + c;
-#pragma unroll
-                for (int m = 0; m < 16; ++m)
-                    if (m < nrow) gp[4 * m * Wd] = sa[r0 + 4 * m][c];
-            }
-            continue;   // the next tile's list building passes two barriers before sa is rewritten
         }
         if (!cols_in) continue;
 #pragma unroll
@@ -489,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels_kernel(const __grid_co
 }  // namespace
 
 cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long pixel_tiles, int max_image_tiles,
-                            cudaStream_t s) {
+                            int ndim_mask, cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
     const size_t smem1 = codebook_smem_floats(max_M) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(bwd_codebook_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
@@ -498,24 +549,29 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
     bwd_codebook_kernel<<<B, B <= kSoloImages ? kCodebookThreads : kRunThreads, smem1, s>>>(L);
     e = cudaGetLastError();
     if (e != cudaSuccess || !L.grad_h || pixel_tiles <= 0) return e;
-    const size_t smem2 = (size_t)max_M * (16 + 7 * sizeof(int));   // list records, positions, sites, tile list
-    e = cudaFuncSetAttribute(bwd_pixels_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-    if (e != cudaSuccess) return e;
-    // one CTA per image when the batch fills the GPU; otherwise each image's tiles are shared out
-    // over `split` CTAs (a single large image would else run on one SM)
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_pixels_kernel, kThreads, smem2)) != cudaSuccess)
-        return e;
-    const long long slots = (long long)sms * (per_sm > 0 ? per_sm : 1);
-    long long split = (slots + B - 1) / B;
-    if (split > max_image_tiles) split = max_image_tiles;
-    if (split < 1) split = 1;
-    BackwardLaunch L2 = L;
-    L2.split = (int)split;
-    bwd_pixels_kernel<<<(unsigned)(B * split), kThreads, smem2, s>>>(L2);
-    return cudaGetLastError();
+    // each image's tiles are shared out over `split` CTAs: as many as fill the GPU, and up to `waves` times
+    // that while an image's CTAs still have four times a tile for each warp (a batch's large images then
+    // end together, and neighbouring tiles run at the same time: 4096 ragged images 541 us with a CTA each,
+    // 514 with two; 256 of 512 x 512 127 us with three, 86 with sixteen)
+    auto launch = [&](auto* kernel, int threads, size_t smem, long long waves, long long most) {
+        int per_sm = 0;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+        if (e != cudaSuccess) return;
+        const long long slots = (long long)sms * std::max(per_sm, 1);
+        BackwardLaunch L2 = L;
+        L2.split = (int)std::max({1LL, std::min((slots + B - 1) / B, most), waves > 1 ? std::min((slots * waves + B - 1) / B, most / 4) : 1LL});
+        kernel<<<(unsigned)(B * (long long)L2.split), threads, smem, s>>>(L2);
+        e = cudaGetLastError();
+    };
+    if (ndim_mask & 4)
+        launch(bwd_pixels2d_kernel, 32 * kPixWarps, (size_t)max_M * sizeof(float4), 6, max_image_tiles);
+    if (e == cudaSuccess && (ndim_mask & 8))   // list records, positions, sites, tile list
+        launch(bwd_pixels3d_kernel, kThreads, (size_t)max_M * (16 + 7 * sizeof(int)), 1, max_image_tiles);
+    return e;
 }
 
 }  // namespace itc

@@ -305,5 +305,5 @@ cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
 // max_blocks: most 64 x 64 pixel blocks of one image; kinds: bit kSeg* for each kind of image in the plan
 cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int kinds, cudaStream_t s);
 cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long pixel_tiles, int max_image_tiles,
-                            cudaStream_t s);
+                            int ndim_mask, cudaStream_t s);
 }  // namespace itc
