@@ -268,8 +268,9 @@ int itc_plan_offsets(const void* plan_host, int b, size_t* field_off, size_t* w_
  * itc_run -- Algorithm 1 for every image of a plan: fields (step 2) for all images in one
  * launch per parameter class, then all images' iterations (steps 3-11) in one launch per
  * lattice dimension: a CTA per image with more than 64 codebook vectors, smaller images 2, 4 or
- * 8 to a CTA, each stopping on its own (the results equal those of one image per CTA bit for
- * bit).  W is read as the initial codebooks (step 1 is done by the caller) and overwritten
+ * 8 to a CTA in large batches, and images with more than 128 vectors on a cluster of up to 8 CTAs
+ * where there are few (a launch of its own); each image stops on its own (the results are the same
+ * bit for bit however the images are grouped).  W is read as the initial codebooks (step 1 is done by the caller) and overwritten
  * with the result.  The fields stay in `ws` for a following itc_backward with the same plan.
  *   plan_host, plan_dev : the same plan bytes on host and on device
  *   W      : device ragged [sum M][ndim], in/out
@@ -349,11 +350,11 @@ int itc_autotune(void* plan_host, void* plan_dev, void* ws, size_t ws_bytes, int
 
 /*
  * itc_plan_configure -- set the fields-pass configuration of class c by hand (what itc_autotune
- * chooses): staging 1 = tensor tiles with tile_h 32, 64 or 128 output rows, staging 0 = plain loads
- * with the fixed tile height of the lattice dimension (64 in 2-D, 32 in 3-D; pass it);
+ * chooses): staging 1 = tensor tiles with tile_h 64 output rows (or 32 or 128 for radii 6, 9 and 12),
+ * staging 0 = thread loads (any row alignment) with the fixed tile height of the lattice dimension (64 in 2-D, 32 in 3-D; pass it);
  * grid_per_sm = persistent CTAs per SM (0 = as many as fit, else 1..64).  Updates the host
  * plan and copies it to plan_dev (synchronously on `stream`).  Errors: ITC_ERR_INVALID_ARG,
- * ITC_ERR_UNSUPPORTED (tensor tiles for a class whose images cannot use them, or a
+ * ITC_ERR_UNSUPPORTED (tensor tiles for a class whose images or radius cannot use them, or a
  * self-overlap class), ITC_ERR_CUDA.
  */
 int itc_plan_configure(void* plan_host, void* plan_dev, int c, int tile_h, int grid_per_sm,

@@ -8,7 +8,7 @@
 // order with one rounding each, no fused multiply-add), lowest k on ties; pixels without data
 // get -1.
 //
-// A warp takes 64 x 64 pixel blocks in turn, each on its own (no block-wide barrier after the sites are
+// A warp takes 64 x 64 pixel blocks (16 x 64 where there are few) in turn, each on its own (no block-wide barrier after the sites are
 // staged): the block's data as bit masks first, one column of each half per lane, so that blocks
 // and 16 x 16 tiles without data only write -1.  For the others the codebooks that can win somewhere
 // are listed, first for the block and from that list for each tile: with dmin_k / dmax_k the metric
@@ -17,8 +17,10 @@
 // order, so the first strict minimum over one is the lowest index on ties.  A lane then takes 8 rows
 // of one column: the column's term once per codebook, the rows' terms and sums as packed operations.
 // Bound by instruction issue (the bytes take 38 us).  1024 ragged shapes (64 to 512 px a side, M 16 to
-// 128, 84 Mpx): 0.67 -> 0.19 ms; before, every 16 x 16 tile listed from the whole codebook, with or
+// 128, 84 Mpx): 0.67 -> 0.18 ms; before, every 16 x 16 tile listed from the whole codebook, with or
 // without data, and each pixel ran through its list in integers.
+#include <algorithm>
+
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -83,17 +85,19 @@ __device__ __forceinline__ int list_box(const SegSmem& S, const unsigned short* 
     return nl;
 }
 
-// The blocks t0, t0 + step, .. of one image.  T: type of the data that says where the image has some.
+// The blocks (bh rows, 64 or 16) t0, t0 + step, .. of one image.  T: type of the data that says where the image has some.
 template <int ND, typename T>
 __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data, const SegSmem& S, short* out, int t0,
-                                               int step, const float (&q)[3]) {
+                                               int step, int bh, const float (&q)[3]) {
     const int lane = threadIdx.x & 31, c = lane & 15, r0 = (lane >> 4) * kSegRows;   // column, first row in a tile
     const int H = D.H, Wd = D.W, G = D.G, pitch = D.pitch, M = D.M;
     const unsigned char* gray = reinterpret_cast<const unsigned char*>(D.data);   // 3-D
-    const int blocks_v = (Wd + kSegBlock - 1) / kSegBlock, nblocks = blocks_v * ((H + kSegBlock - 1) / kSegBlock);
+    const int blocks_v = (Wd + kSegBlock - 1) / kSegBlock, nblocks = blocks_v * ((H + bh - 1) / bh);
     for (int t = t0; t < nblocks; t += step) {
-        const int ub = (t / blocks_v) * kSegBlock, vb = (t % blocks_v) * kSegBlock;
-        int nb = -1;   // the block's list is made when a tile needs it
+        const int ub = (t / blocks_v) * bh, vb = (t % blocks_v) * kSegBlock;
+        // the block's list is made when a tile needs it; up to 32 vectors are a step of the tile's own list
+        int nb = M <= 32 ? M : -1;
+        const unsigned short* from = M <= 32 ? nullptr : S.block;
         for (int half = 0; half < 2; ++half) {
             const int vh = vb + 32 * half;
             if (vh >= Wd) break;
@@ -105,6 +109,7 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
                 for (int w = 0; w < 2; ++w) {
 #pragma unroll
                     for (int p = 0; p < 32; p += 16) {
+                        if (32 * w + p >= bh) break;
                         T x[16];
 #pragma unroll
                         for (int r = 0; r < 16; ++r) x[r] = __ldg(col + (size_t)min(ub + 32 * w + p + r, H - 1) * pitch);
@@ -117,7 +122,7 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
             }
             if (vh + lane >= Wd) mask[0] = mask[1] = 0u;
 #pragma unroll 1
-            for (int s = 0; s < 2 * (kSegBlock / kSegTile); ++s) {
+            for (int s = 0; s < bh / kSegTile * 2; ++s) {
                 const int rb = s >> 1, co = (s & 1) * kSegTile;
                 const int ut = ub + rb * kSegTile, v0 = vh + co, v = v0 + c, u0 = ut + r0;
                 if (ut >= H || v0 >= Wd) continue;
@@ -133,12 +138,12 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
                     continue;
                 }
                 if (nb < 0)
-                    nb = list_box<ND>(S, nullptr, M, S.block, ub, min(ub + kSegBlock, H) - 1, vb, min(vb + kSegBlock, Wd) - 1,
+                    nb = list_box<ND>(S, nullptr, M, S.block, ub, min(ub + bh, H) - 1, vb, min(vb + kSegBlock, Wd) - 1,
                                       G, q);
                 // the box of the tile's data: rows and columns with any
                 const unsigned rows = __reduce_or_sync(kFull, on << r0), cols2 = __ballot_sync(kFull, on != 0u);
                 const unsigned cols = (cols2 | (cols2 >> 16)) & 0xffffu;
-                const int nl = list_box<ND>(S, S.block, nb, S.tile, ut + __ffs(rows) - 1, ut + 31 - __clz(rows),
+                const int nl = list_box<ND>(S, from, nb, S.tile, ut + __ffs(rows) - 1, ut + 31 - __clz(rows),
                                             v0 + __ffs(cols) - 1, v0 + 31 - __clz(cols), G, q);
                 float fg[ND == 3 ? kSegRows : 1];
                 if constexpr (ND == 3) {
@@ -194,7 +199,7 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
 // split CTAs per image: their warps share out its blocks.  KIND: the images of the launch, bytes, weights or
 // gray (others return).
 template <int KIND>
-__global__ void __launch_bounds__(kSegThreads, 5) segment_kernel(const __grid_constant__ SegmentLaunch L) {
+__global__ void __launch_bounds__(kSegThreads, KIND == kSegGray ? 4 : 5) segment_kernel(const __grid_constant__ SegmentLaunch L) {
     const int img = __ldg(L.order + blockIdx.x / L.split), part = blockIdx.x % L.split;
     const ImageDesc& D = L.descs[img];
     constexpr int nd = KIND == kSegGray ? 3 : 2;
@@ -202,7 +207,10 @@ __global__ void __launch_bounds__(kSegThreads, 5) segment_kernel(const __grid_co
     const int M = D.M, tid = threadIdx.x, wid = tid >> 5, nw = kSegThreads / 32;
     const int blocks = D.bwd_tiles_u * D.bwd_tiles_v;
     static_assert(kSegBlock == kBwdTileH && kSegBlock == kBwdTileW, "blocks are the backward's tiles");
-    if (part * nw >= blocks) return;
+    // strips of 16 rows where there are few blocks for the image's warps: 770 images of up to 67 px with 8
+    // vectors, whose one block would keep one warp, take 16 us instead of 25
+    const int step = L.split * nw, bh = blocks < 2 * step ? kSegTile : kSegBlock;
+    if (part * nw >= (bh == kSegTile ? D.bwd_tiles_v * ((D.H + kSegTile - 1) / kSegTile) : blocks)) return;
     // q_i = 1 / tau_i^2: the square of the float width in double (exact), one division, one
     // rounding to float
     float q[3];
@@ -221,10 +229,10 @@ __global__ void __launch_bounds__(kSegThreads, 5) segment_kernel(const __grid_co
     }
     __syncthreads();
     short* out = L.labels + D.gh_off;
-    const int t0 = part * nw + wid, step = L.split * nw;
-    if constexpr (KIND == kSegGray) segment_blocks<3, float>(D, D.weight, S, out, t0, step, q);
-    else if constexpr (KIND == kSegBytes) segment_blocks<2>(D, reinterpret_cast<const unsigned char*>(D.data), S, out, t0, step, q);
-    else segment_blocks<2>(D, reinterpret_cast<const float*>(D.data), S, out, t0, step, q);
+    const int t0 = part * nw + wid;
+    if constexpr (KIND == kSegGray) segment_blocks<3, float>(D, D.weight, S, out, t0, step, bh, q);
+    else if constexpr (KIND == kSegBytes) segment_blocks<2>(D, reinterpret_cast<const unsigned char*>(D.data), S, out, t0, step, bh, q);
+    else segment_blocks<2>(D, reinterpret_cast<const float*>(D.data), S, out, t0, step, bh, q);
 }
 
 template <int KIND>
@@ -233,11 +241,15 @@ cudaError_t launch_kind(const SegmentLaunch& L, int B, int max_M, int max_blocks
     cudaError_t e = cudaFuncSetAttribute(segment_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // a large image is shared out over several CTAs, eight blocks a warp (four: 5 % slower, more CTAs stage
-    // the sites), or one where the batch does not fill the GPU (152 SMs, five CTAs each)
-    const int nw = kSegThreads / 32;
-    const int per = B < 152 * 5 ? 1 : 8;
+    // the sites).  A batch that does not fill the GPU (152 SMs, five CTAs each) takes a block a warp, two if
+    // that makes many CTAs, and as few as a strip while it leaves SMs without work (300 ragged images 86 ->
+    // 64 us, 42 of 500 px with 327 vectors 75 -> 49, one of 300 px 19 -> 7).
+    const int nw = kSegThreads / 32, slots = 152 * 5;
+    auto ctas = [&](int blocks_per_warp) { return (max_blocks + blocks_per_warp * nw - 1) / (blocks_per_warp * nw); };
     SegmentLaunch L2 = L;
-    L2.split = (max_blocks + per * nw - 1) / (per * nw);
+    if (B >= slots) L2.split = ctas(8);
+    else if ((long long)B * ctas(1) >= 4 * slots) L2.split = ctas(2);
+    else L2.split = std::max(ctas(1), std::min((kSegBlock / kSegTile * max_blocks + nw - 1) / nw, slots / B));
     segment_kernel<KIND><<<(unsigned)(B * L2.split), kSegThreads, smem, s>>>(L2);
     return cudaGetLastError();
 }

@@ -55,3 +55,16 @@ def test_blocks_3d(weighted):
     for b, (im, W, lab) in enumerate(zip(images, books, got)):
         ref = oracle.segment3d(im, sigma, W, 50, weights[b] if weighted else None)
         assert np.array_equal(lab.astype(np.int32), ref), im.shape
+
+
+@pytest.mark.parametrize("large", [(70, 520), (300, 280)])
+def test_blocks_of_a_large_batch(large):
+    """Enough images to fill the GPU: whole blocks for the large ones, strips of 16 rows for the small."""
+    rng = np.random.default_rng(large[0])
+    shapes = [(int(a), int(b)) for a, b in rng.integers(3, 40, (790, 2))] + [large] * 3 + [(64, 64), (65, 129)]
+    images = [(rng.random(s) < 0.5).astype(np.uint8) for s in shapes]
+    books = [np.stack([rng.uniform(-1, s[0], m), rng.uniform(-1, s[1], m)], 1).astype(np.float32)
+             for s, m in zip(shapes, rng.integers(1, 40, len(shapes)))]
+    got = _labels(images, books, 2.7)
+    for b in [*range(0, 790, 40), *range(790, len(shapes))]:
+        assert np.array_equal(got[b].astype(np.int32), oracle.segment2d(images[b], 2.7, books[b])), shapes[b]
