@@ -38,8 +38,8 @@ FALLBACK_HBM_GBS = 6800.0
 # profiles/fields3d_kernel_c5_gray3d.md), valid only for the kernel source it was taken on
 # (sha256 prefix below); scaled to a launch by its site count (pixels, or voxels of the 3-D lattice).
 FIELDS_TRAFFIC = {
-    "c3": {"bytes_per_site": 969.25e6 / 86358723, "source_sha256": "c1919dae6100b141",
-           "source": "paper_1310_7114_gb300/csrc/itc_fields_tma.cu",
+    "c3": {"bytes_per_site": 968.86e6 / 86358723, "source_sha256": "2219d1a8248e79c7",
+           "source": "paper_1310_7114_gb300/csrc/itc_fields_tma.cuh",
            "note": "ncu dram bytes of the 1024-image capture scaled by pixels (profiles/fields_tma_kernel_c3_1024.md)"},
     "c5": {"bytes_per_site": (0.27e6 + 206.93e6) / 16777216, "source_sha256": "6eedaafde8ac4a48",
            "source": "paper_1310_7114_gb300/csrc/itc_fields3d.cu",
@@ -64,7 +64,7 @@ def fields_kernel_name(ndims, tuning):
     if all(d == 3 for d in ndims):
         return "fields3d_kernel (persistent CTAs over runs of one-slice tiles, one launch)"
     kinds = sorted({c["staging"] for c in tuning})
-    names = {"tma": "fields_tma_kernel", "plain": "fields_kernel"}
+    names = {"tma": "fields_tma_kernel", "plain": "fields_tma_kernel (thread staging) or fields_kernel"}
     return " + ".join(names.get(k, k) for k in kinds) + " (persistent, one launch per sigma class)"
 
 WORKLOADS = {
