@@ -10,7 +10,7 @@
 // window sums around round(w_k) read directly from the image (kernel evaluated at the real w_k, one
 // warp per k), the M x M sums s_k, E_k (one thread per k), S_XW, S_WW, grad_W and two per-image
 // scalars for kernel 2.
-// Kernel 2 (per dimension; 16 x 64 pixel tiles of a warp in 2-D, 64 x 64 of a CTA in 3-D): the codebooks
+// Kernel 2 (per dimension; 16 x 64 pixel tiles of a warp in 2-D, 32 x 32 or 16 x 16 of a CTA in 3-D): the codebooks
 // whose box meets a tile are taken in k order (ballots), their Gaussians are stamped onto the tile in
 // that order -- the transposed form of the gather in the forward update -- and every pixel
 // combines the stored field A with the stamp.
@@ -385,10 +385,13 @@ __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const _
 
 constexpr int kChunk = 64;   // codebooks staged per round in the 3-D pixel kernel
 
-// 3-D pixel pass: one CTA per image walks the image's 64 x 64 tiles (images with the most tiles
-// are launched first).  The codebooks whose box meets a tile are listed in k order; chunks of 64 of them are
-// staged as a (64 x 64) and b (64 x 64) in shared memory and every thread accumulates a 4 x 4 block of pixels
-// in l order.  The g factor depends on each pixel's gray level and is applied per pixel and codebook.
+// 3-D pixel pass: a CTA walks T x T tiles of its image (images with the most tiles are launched first).  The
+// codebooks whose box meets the tile are listed in k order; chunks of 64 of them are staged as a (64 x T) and
+// b (64 x T) in shared memory and every thread accumulates a T / 16 square of pixels in l order.  The g factor
+// depends on each pixel's gray level and is applied per pixel and codebook, so the pass is bound by its chain
+// of exponentials where there are few pixels.  T = 32, or 16 where tiles of 32 would not fill the GPU: one
+// 256 x 256 image with 64 vectors 21 us at T = 64, 6.4 at 32, 4.5 at 16; 16 of them 31, 20 and 29.
+template <int T>
 __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_constant__ BackwardLaunch L) {
     // split CTAs per image (few large images): CTA s of an image takes its tiles s, s + split, ...
     const int split = L.split;
@@ -397,8 +400,8 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
     const ImageDesc& D = L.descs[img];
     if (D.ndim != 3) return;
     const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int H = D.H, Wd = D.W, G = D.G, fpitch = D.fpitch, tiles_v = D.bwd_tiles_v;
-    const int ntiles = D.bwd_tiles_u * D.bwd_tiles_v;
+    const int H = D.H, Wd = D.W, G = D.G, fpitch = D.fpitch, tiles_v = (Wd + T - 1) / T;
+    const int ntiles = tiles_v * ((H + T - 1) / T);
     const int Ru = D.R[0], Rv = D.R[1], Rg = D.R[2];
     const float c0 = D.inv2s2[0], c1 = D.inv2s2[1], c2 = D.inv2s2[2];
     // the separable factors exp(-d^2 c) = 2^(-d^2 c log2 e), log2 e folded into the widths
@@ -414,8 +417,8 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
     float* cw = reinterpret_cast<float*>(lc + M);       // M x 3 codebook positions
     int* cr = reinterpret_cast<int*>(cw + 3 * M);       // M x 3 rounded lattice sites
     int* lk = cr + 3 * M;                               // listed codebooks of the current tile
-    __shared__ __align__(16) float sa[kChunk][kBwdTileH];
-    __shared__ __align__(16) float sb[kChunk][kBwdTileW];
+    __shared__ __align__(16) float sa[kChunk][T];
+    __shared__ __align__(16) float sb[kChunk][T];
     __shared__ __align__(16) int wcount[kThreads / 32];
 
     const float* Wk = L.W + D.w_off;
@@ -430,16 +433,17 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
     }
     __syncthreads();
 
-    const int pr = (tid >> 4) * 4, pc = (tid & 15) * 4;   // this thread's 4 x 4 block
+    constexpr int P = T / 16;   // this thread's P x P block
+    const int pr = (tid >> 4) * P, pc = (tid & 15) * P;
     if (part >= ntiles) return;
     for (int t = part; t < ntiles; t += split) {
-        const int u0 = (t / tiles_v) * kBwdTileH, v0 = (t % tiles_v) * kBwdTileW;
-        int gray[4][4];
+        const int u0 = (t / tiles_v) * T, v0 = (t % tiles_v) * T;
+        int gray[P][P];
         const bool cols_in = v0 + pc < Wd;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < P; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < P; ++j) {
                 const int u = u0 + pr + i, v = v0 + pc + j;
                 gray[i][j] = (u < H && v < Wd) ? pixel_gray(D, u, v) : 0;
             }
@@ -451,8 +455,8 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
             bool hit = false;
             if (k < M) {
                 const int r0 = cr[k * 3], r1 = cr[k * 3 + 1];
-                hit = (r0 + Ru >= u0) && (r0 - Ru <= u0 + kBwdTileH - 1) &&
-                      (r1 + Rv >= v0) && (r1 - Rv <= v0 + kBwdTileW - 1);
+                hit = (r0 + Ru >= u0) && (r0 - Ru <= u0 + T - 1) &&
+                      (r1 + Rv >= v0) && (r1 - Rv <= v0 + T - 1);
             }
             const unsigned bal = __ballot_sync(0xffffffffu, hit);
             if (lane == 0) wcount[wid] = __popc(bal);
@@ -475,11 +479,11 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
             __syncthreads();
         }
 
-        float acc[4][4] = {};
+        float acc[P][P] = {};
         // factor staging: each thread fills one row / column r of the factors for every fourth l
-        const int sr = tid & (kBwdTileH - 1), sl = tid / kBwdTileH;
-        static_assert(kBwdTileH == kBwdTileW && kThreads % kBwdTileH == 0, "square tiles, whole rows of threads");
-        constexpr int kStageStep = kThreads / kBwdTileH;
+        const int sr = tid & (T - 1), sl = tid / T;
+        static_assert(kThreads % T == 0, "whole rows of threads");
+        constexpr int kStageStep = kThreads / T;
         const int su = u0 + sr, sv = v0 + sr;
         const bool su_in = su < H, sv_in = sv < Wd;
         const float fu = (float)su, fv = (float)sv;
@@ -495,16 +499,19 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
             }
             __syncthreads();
             for (int l = 0; l < nc; ++l) {
-                const float4 av4 = *reinterpret_cast<const float4*>(&sa[l][pr]);
-                const float4 bv4 = *reinterpret_cast<const float4*>(&sb[l][pc]);
-                const float av[4] = {av4.x, av4.y, av4.z, av4.w}, bv[4] = {bv4.x, bv4.y, bv4.z, bv4.w};
+                float av[P], bv[P];
+#pragma unroll
+                for (int i = 0; i < P; ++i) {
+                    av[i] = sa[l][pr + i];
+                    bv[i] = sb[l][pc + i];
+                }
                 const int k = lk[base + l];
                 const float wg = cw[k * 3 + 2];
                 const int rg = cr[k * 3 + 2];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < P; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < P; ++j) {
                         const int gl = gray[i][j];
                         if (abs(gl - rg) <= Rg) {
                             const float d = (float)gl - wg;
@@ -516,13 +523,13 @@ __global__ void __launch_bounds__(kThreads, 3) bwd_pixels3d_kernel(const __grid_
         }
         if (!cols_in) continue;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < P; ++i) {
             const int u = u0 + pr + i;
             if (u >= H) break;
             float* out = gh + (long long)u * Wd + v0 + pc;
             {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < P; ++j) {
                     const int v = v0 + pc + j;
                     if (v >= Wd) break;
                     if (gray[i][j] >= G) {   // a voxel outside the lattice: no field value
@@ -569,8 +576,11 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
     };
     if (ndim_mask & 4)
         launch(bwd_pixels2d_kernel, 32 * kPixWarps, (size_t)max_M * sizeof(float4), 6, max_image_tiles);
-    if (e == cudaSuccess && (ndim_mask & 8))   // list records, positions, sites, tile list
-        launch(bwd_pixels3d_kernel, kThreads, (size_t)max_M * (16 + 7 * sizeof(int)), 1, max_image_tiles);
+    if (e == cudaSuccess && (ndim_mask & 8)) {   // list records, positions, sites, tile list
+        const size_t smem = (size_t)max_M * (16 + 7 * sizeof(int));
+        if (4 * pixel_tiles < 3LL * sms) launch(bwd_pixels3d_kernel<16>, kThreads, smem, 1, 16LL * max_image_tiles);
+        else launch(bwd_pixels3d_kernel<32>, kThreads, smem, 1, 4LL * max_image_tiles);
+    }
     return e;
 }
 

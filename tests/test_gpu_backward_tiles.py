@@ -56,3 +56,15 @@ def test_mixed_dimensions():
     for b in range(4):
         gW1, gh1 = _grads(images[b:b + 1], books[b:b + 1], 2.0, ndims[b:b + 1], Gs[b:b + 1])
         assert np.array_equal(gW[b], gW1[0]) and np.array_equal(gh[b], gh1[0]), b
+
+
+@pytest.mark.parametrize("shape", [(260, 250), (257, 289)])
+def test_gray_tiles(shape):
+    """A batch that fills the GPU takes larger tiles than one image: the same gradients, bit for bit."""
+    rng = np.random.default_rng(shape[1])
+    images = [rng.integers(0, 12, shape).astype(np.uint8) for _ in range(8)]
+    books = [(rng.random((70, 3)) * (np.array([*shape, 12]) - 1)).astype(np.float32) for _ in images]
+    gW, gh = _grads(images, books, (2.0, 3.0, 2.0), [3] * 8, [12] * 8)
+    for b in (0, 7):
+        gW1, gh1 = _grads(images[b:b + 1], books[b:b + 1], (2.0, 3.0, 2.0), [3], [12])
+        assert np.array_equal(gW[b], gW1[0]) and np.array_equal(gh[b], gh1[0]), b
