@@ -30,6 +30,7 @@
 #pragma once
 #include <cuda.h>
 
+#include "itc_bytes.cuh"
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -202,7 +203,8 @@ struct TmaTile {
                                                : 2 * (size_t)STAGE_BYTES;
     // byte inputs with centred moments and R >= 9 take row windows that are one run of 0/1 inputs
     // from a table (below), where the launch has tiles enough to repay building it; it does not fit
-    // beside 128-row tiles at R = 12, and a window is a word of bits up to R = 13
+    // beside 128-row tiles at R = 12, and the 4 + 2R inputs of an item are a word of bits up to R = 13
+    // (there 2048 ragged silhouettes take 802 us with the table and 831 without)
     static constexpr bool RUNS = LM != kFew && DTYPE == ITC_U8 && !ABS && R >= 9 && R <= 13 && !(TH == 128 && R == 12);
     static constexpr int NTAP = 2 * R + 1;
     static constexpr int T2 = (NTAP + 1) * (NTAP + 2) / 2;             // runs [a, b), 0 <= a <= b <= NTAP
@@ -672,19 +674,13 @@ __global__ void __launch_bounds__(kThreads, (TmaTile<R, ABS, DTYPE, TH, AO, STG,
                     return false;
                 } else {
                     constexpr int N = TT::NTAP;
-                    constexpr uint32_t FULL = (1u << NW4) - 1u;     // NW4 <= 28
+                    constexpr uint32_t FULL = (1u << NW4) - 1u;     // NW4 <= 30
                     constexpr uint32_t EDGES = (1u << (NW4 - 1)) - 1u;
-                    uint32_t high = 0u, m0 = 0u, m1 = 0u;
+                    uint32_t high = 0u;
 #pragma unroll
-                    for (int q = 0; q < NQ4; ++q) {
-                        high |= (w0[q] | w1[q]) & (0xfefefefeu & window_mask<OFF, NW4>(q));
-                        // the low bits of the 4 bytes gathered into 4 bits (no carries: the 16
-                        // partial products land on distinct bits)
-                        m0 |= (((w0[q] & 0x01010101u) * 0x01020408u) >> 24) << (4 * q);
-                        m1 |= (((w1[q] & 0x01010101u) * 0x01020408u) >> 24) << (4 * q);
-                    }
-                    m0 = (m0 >> OFF) & FULL;   // bit i: input at column c - R + i
-                    m1 = (m1 >> OFF) & FULL;
+                    for (int q = 0; q < NQ4; ++q) high |= (w0[q] | w1[q]) & (0xfefefefeu & window_mask<OFF, NW4>(q));
+                    const uint32_t m0 = window_bits<OFF, NW4>(w0);   // bit i: input at column c - R + i
+                    const uint32_t m1 = window_bits<OFF, NW4>(w1);
                     if (high != 0u || __popc((m0 ^ (m0 >> 1)) & EDGES) > 2 || __popc((m1 ^ (m1 >> 1)) & EDGES) > 2)
                         return false;
                     const int r0 = (item >> 4) * 2, c = (item & 15) * 4;
