@@ -550,7 +550,7 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
                             int ndim_mask, cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
     const size_t smem1 = codebook_smem_floats(max_M) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(bwd_codebook_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+    cudaError_t e = allow_smem(bwd_codebook_kernel, codebook_smem_floats(ITC_MAX_M) * sizeof(float));
     if (e != cudaSuccess) return e;
     // few images: as many threads as keep a CTA's window sums and pair sums short
     bwd_codebook_kernel<<<B, B <= kSoloImages ? kCodebookThreads : kRunThreads, smem1, s>>>(L);
@@ -563,9 +563,10 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
     // that while an image's CTAs still have four times a tile for each warp (a batch's large images then
     // end together, and neighbouring tiles run at the same time: 4096 ragged images 541 us with a CTA each,
     // 514 with two; 256 of 512 x 512 127 us with three, 86 with sixteen)
-    auto launch = [&](auto* kernel, int threads, size_t smem, long long waves, long long most) {
+    auto launch = [&](auto* kernel, int threads, size_t per_vector, long long waves, long long most) {
         int per_sm = 0;
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const size_t smem = (size_t)max_M * per_vector;
+        e = allow_smem(kernel, ITC_MAX_M * per_vector);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
         if (e != cudaSuccess) return;
         const long long slots = (long long)sms * std::max(per_sm, 1);
@@ -575,11 +576,11 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
         e = cudaGetLastError();
     };
     if (ndim_mask & 4)
-        launch(bwd_pixels2d_kernel, 32 * kPixWarps, (size_t)max_M * sizeof(float4), 6, max_image_tiles);
+        launch(bwd_pixels2d_kernel, 32 * kPixWarps, sizeof(float4), 6, max_image_tiles);
     if (e == cudaSuccess && (ndim_mask & 8)) {   // list records, positions, sites, tile list
-        const size_t smem = (size_t)max_M * (16 + 7 * sizeof(int));
-        if (4 * pixel_tiles < 3LL * sms) launch(bwd_pixels3d_kernel<16>, kThreads, smem, 1, 16LL * max_image_tiles);
-        else launch(bwd_pixels3d_kernel<32>, kThreads, smem, 1, 4LL * max_image_tiles);
+        constexpr size_t per_vector = 16 + 7 * sizeof(int);
+        if (4 * pixel_tiles < 3LL * sms) launch(bwd_pixels3d_kernel<16>, kThreads, per_vector, 1, 16LL * max_image_tiles);
+        else launch(bwd_pixels3d_kernel<32>, kThreads, per_vector, 1, 4LL * max_image_tiles);
     }
     return e;
 }

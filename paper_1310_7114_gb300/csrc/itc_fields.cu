@@ -303,13 +303,14 @@ __global__ void __launch_bounds__(kThreads, 2) fields_kernel(const __grid_consta
 
 template <int RU, int RV, bool ABS, int DTYPE, int TH>
 cudaError_t launch_one(const FieldsLaunch& L, int nblocks, int Ru, int Rv, cudaStream_t s) {
-    const int rows = TH + 2 * Ru;
-    const int SW = ((kTileW + 2 * Rv + 3) & ~3) + 4;
-    const size_t smem = (size_t)rows * SW * sizeof(float) + (size_t)2 * rows * kTileW * sizeof(float);
+    auto smem = [](int ru, int rv) {
+        const int rows = TH + 2 * ru, SW = ((kTileW + 2 * rv + 3) & ~3) + 4;
+        return (size_t)rows * SW * sizeof(float) + (size_t)2 * rows * kTileW * sizeof(float);
+    };
     auto k = fields_kernel<RU, RV, ABS, DTYPE, TH>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, RU > 0 ? smem(RU, RV) : smem(ITC_MAX_RADIUS_UV, ITC_MAX_RADIUS_UV));
     if (e != cudaSuccess) return e;
-    k<<<nblocks, kThreads, smem, s>>>(L);
+    k<<<nblocks, kThreads, smem(Ru, Rv), s>>>(L);
     return cudaGetLastError();
 }
 

@@ -402,12 +402,14 @@ __global__ void __launch_bounds__(kThreads, (RU > 0 && RU <= 9) ? 3 : 2) fields3
 
 template <int RU, int RV, bool ABS, int TH>
 cudaError_t launch_3d(const FieldsLaunch& L, int ntiles, int Ru, int Rv, cudaStream_t s) {
-    const int rows = TH + 2 * Ru;
-    const int SW = (kTileW + 2 * Rv + 3) & ~3;
-    const size_t smem = ((size_t)2 * rows * SW + (size_t)3 * rows * kTileW + ((2 * L.taps.R[2] + 4) & ~3)) * sizeof(float) +
-                        (size_t)rows * SW;   // S, S_g, T, T_v, T_g, the g taps, the gray bytes
+    auto bytes = [](int ru, int rv, int rg) {   // S, S_g, T, T_v, T_g, the g taps, the gray bytes
+        const int rows = TH + 2 * ru, SW = (kTileW + 2 * rv + 3) & ~3;
+        return ((size_t)2 * rows * SW + (size_t)3 * rows * kTileW + ((2 * rg + 4) & ~3)) * sizeof(float) + (size_t)rows * SW;
+    };
+    const size_t smem = bytes(Ru, Rv, L.taps.R[2]);
     auto k = fields3d_kernel<RU, RV, ABS, TH>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, RU > 0 ? bytes(RU, RV, ITC_MAX_RADIUS_G)
+                                         : bytes(ITC_MAX_RADIUS_UV_3D, ITC_MAX_RADIUS_UV_3D, ITC_MAX_RADIUS_G));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

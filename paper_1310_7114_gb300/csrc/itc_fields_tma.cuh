@@ -861,7 +861,7 @@ cudaError_t launch_tma(const FieldsLaunch& L, int ntiles, cudaStream_t s) {
     using TT = TmaTile<R, ABS, DTYPE, TH, AO, STG, LM>;
     const size_t smem = TT::SMEM;
     auto k = fields_tma_kernel<R, ABS, DTYPE, TH, AO, STG, LM>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     static ResidentCtas resident;
     int sms = 0, per_sm = 0;

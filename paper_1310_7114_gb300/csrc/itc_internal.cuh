@@ -165,6 +165,14 @@ struct ResidentCtas {
     }
 };
 
+// Allows a kernel `most` bytes of dynamic shared memory, the most that any call of it takes.  The limit is one
+// for all host threads: set to a call's own size, another thread's smaller call could lower it before the
+// launch, which then fails.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Tile height of the fields kernels for a given radius (rows of outputs per CTA).

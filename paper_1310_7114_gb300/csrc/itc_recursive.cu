@@ -615,8 +615,9 @@ static cudaError_t launch_scan(const RecursiveLaunch& L, int nimg, int max_H, in
     max_H = max_H < kRecMaxLine ? max_H : kRecMaxLine;
     max_W = max_W < kRecMaxLine ? max_W : kRecMaxLine;
     auto go = [&](auto k, int nlines, int len, int arrays) -> cudaError_t {
-        const size_t smem = (size_t)kRecPairs * rec_pair_floats2(len, arrays) * sizeof(float2);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        auto bytes = [&](int n) { return (size_t)kRecPairs * rec_pair_floats2(n, arrays) * sizeof(float2); };
+        const size_t smem = bytes(len);
+        cudaError_t e = allow_smem(k, bytes(kRecMaxLine));
         if (e != cudaSuccess) return e;
         const int nblk = (nlines + kRecLines - 1) / kRecLines;
         k<<<(unsigned)(nimg * nblk), 32 * kRecPairs, smem, s>>>(L, nblk);
@@ -638,10 +639,8 @@ cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int 
     if (e != cudaSuccess || rec_scans(max_H, max_W)) return e;
     // images with a longer side
     const size_t smem = (size_t)kRecRowWarps * kRecTileFloats * sizeof(float);
-    e = cudaFuncSetAttribute(rec_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(rec_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if ((e = allow_smem(rec_rows_kernel<true>, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem(rec_rows_kernel<false>, smem)) != cudaSuccess) return e;
     const dim3 grow((unsigned)nimg, (unsigned)((max_H + 32 * kRecRowWarps - 1) / (32 * kRecRowWarps)));
     const dim3 gcol((unsigned)nimg, (unsigned)((max_W + kRecColThreads - 1) / kRecColThreads));
     if (L.mode == 0) {

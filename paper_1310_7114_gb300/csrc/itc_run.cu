@@ -791,8 +791,7 @@ cudaError_t launch_nd(RunLaunch L, int large_ctas, int nlarge, int ctas, int max
         } else {
             smem = large_smem_floats(max_M, csize, ND) * sizeof(float);
             auto k = csize > 1 ? run_large_kernel<ND, true> : run_large_kernel<ND, false>;
-            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-                return e;
+            if ((e = allow_smem(k, large_smem_floats(ITC_MAX_M, 1, ND) * sizeof(float))) != cudaSuccess) return e;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)(large_ctas * csize));
             cfg.blockDim = dim3((unsigned)large_threads(csize > 1));

@@ -237,8 +237,9 @@ __global__ void __launch_bounds__(kSegThreads, KIND == kSegGray ? 4 : 5) segment
 
 template <int KIND>
 cudaError_t launch_kind(const SegmentLaunch& L, int B, int max_M, int max_blocks, cudaStream_t s) {
-    const size_t smem = (size_t)max_M * (3 * sizeof(float) + 2 * (kSegThreads / 32) * sizeof(unsigned short));
-    cudaError_t e = cudaFuncSetAttribute(segment_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t per_vector = 3 * sizeof(float) + 2 * (kSegThreads / 32) * sizeof(unsigned short);
+    const size_t smem = (size_t)max_M * per_vector;
+    cudaError_t e = allow_smem(segment_kernel<KIND>, ITC_MAX_M * per_vector);
     if (e != cudaSuccess) return e;
     // a large image is shared out over several CTAs, eight blocks a warp (four: 5 % slower, more CTAs stage
     // the sites).  A batch that does not fill the GPU (152 SMs, five CTAs each) takes a block a warp, two if
