@@ -22,4 +22,35 @@ __host__ __device__ __forceinline__ uint32_t window_bits(const uint32_t (&w)[NQ]
     return m & ((1u << N) - 1u);
 }
 
+// Rows on any boundary are read as the aligned 4-byte words that hold their bytes.  A word may hold bytes of
+// the rows around (or the padding between them), but must not reach beyond the image: in row u of H rows of
+// W bytes, `pitch` apart, RowRoom has the bytes of the image before and after the row that a word can reach
+// (up to 3).  A word that begins at column c (a multiple of 4 bytes from a boundary) is taken whole or not at
+// all; row_bytes puts together what is left, the image's first and last bytes.
+struct RowRoom {
+    int before, after;
+    __host__ __device__ __forceinline__ RowRoom(int u, int H, int pitch) {
+        const int p = pitch < 3 ? pitch : 3, a = u < 3 ? u : 3, z = H - 1 - u < 3 ? H - 1 - u : 3;
+        before = a * p < 3 ? a * p : 3;
+        after = z * p < 3 ? z * p : 3;
+    }
+    __host__ __device__ __forceinline__ bool whole(int c, int W) const { return c >= -before && c < W + after - 3; }
+};
+// The same test by the word's offset from the image's first byte, for an image of `bytes` bytes in all.
+struct ByteSpan {
+    unsigned long long last, shift;   // images of less than a word: no offset passes
+    __host__ __device__ __forceinline__ explicit ByteSpan(long long bytes)
+        : last(bytes < 4 ? 0ull : (unsigned long long)bytes - 4), shift(bytes < 4 ? 1ull << 62 : 0ull) {}
+    __host__ __device__ __forceinline__ bool whole_word(long long at) const { return (unsigned long long)at + shift <= last; }
+};
+// the bytes of columns c to c + 3 of a row that lie in words not taken whole (the others: zeros)
+__host__ __device__ __forceinline__ uint32_t row_bytes(const unsigned char* row, int c, int W, const RowRoom& room) {
+    uint32_t w = 0u;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j)
+        if (c + j >= 0 && c + j < W && !room.whole(c + j - (int)(reinterpret_cast<uintptr_t>(row + c + j) & 3), W))
+            w |= (uint32_t)row[c + j] << (8 * j);
+    return w;
+}
+
 }  // namespace itc

@@ -22,6 +22,7 @@
 // down and up again, 4 columns of each 128-column chunk per lane in 32 bits, a scan per chunk and the
 // previous row in shared memory: about 3000 clocks a row of 512 columns; the same two walks with this row
 // layout took 0.34 ms.
+#include "itc_bytes.cuh"
 #include "itc_internal.cuh"
 
 namespace itc {
@@ -31,11 +32,11 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kAhead = 8;   // rows copied ahead (a power of two)
 
 __device__ __forceinline__ unsigned pair16(int a) { return (unsigned)a * 0x00010001u; }
-// asynchronous copies of N bytes to shared memory (zeros if !ok), grouped by row
+// asynchronous copies to shared memory of the first `bytes` of N bytes and zeros, grouped by row
 template <int N>
-__device__ __forceinline__ void copy_async(unsigned* dst, const void* src, bool ok = true) {
+__device__ __forceinline__ void copy_async(unsigned* dst, const void* src, int bytes = N) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(N), "r"(ok ? N : 0) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(N), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void copy_wait_oldest() { asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory"); }
@@ -51,6 +52,14 @@ __device__ __forceinline__ unsigned mask_pair(unsigned lo, unsigned hi, int i, i
 // a value below 2^16 as a float, exactly: the bits of 2^23 + v, minus 2^23
 __device__ __forceinline__ float low_float(unsigned p) { return __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7610)) - 8388608.f; }
 __device__ __forceinline__ float high_float(unsigned p) { return __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7632)) - 8388608.f; }
+
+// The words of a lane's input bytes (columns from j0 on) that reach beyond the image: in its first and last
+// rows, which the two walks start with
+__device__ __noinline__ void first_words(unsigned* dst, int nw, const unsigned char* row, int j0, int W, RowRoom room) {
+    const int c = j0 - (int)(reinterpret_cast<size_t>(row + j0) & 3);
+    for (int q = 0; q <= nw; ++q)
+        if (!room.whole(c + 4 * q, W)) dst[q] = row_bytes(row, c + 4 * q, W, room);
+}
 
 // The warp's rows of one image with up to 32 C columns.  VEC: rows on vector boundaries.  Rows come
 // through a ring in shared memory that each lane fills and reads for itself; copies are unconditional,
@@ -79,25 +88,28 @@ struct Rows {
     __device__ __forceinline__ unsigned* pairs_row(int u) const {
         return reinterpret_cast<unsigned*>(T + (size_t)u * fp) + (in ? lane * R : 0);
     }
-    // the lane's input bytes of row u to the ring; what lies past W is masked later (a vector's bytes past
-    // W lie inside the row's pitch).  Rows without that alignment: the 4-byte words that hold the
-    // bytes, one more than NW, shifted into place when they are read; words past the row are zeros
+    // the lane's input bytes of row u to the ring, zeros past W.  Rows without vector alignment: the 4-byte
+    // words that hold the bytes, one more than NW, shifted into place when they are read; words that reach
+    // beyond the image are left out (first_words)
     __device__ __forceinline__ void copy_in(int u, int t) const {
         const unsigned char* row = X + (size_t)inside(u) * pitch;
         const unsigned char* src = row + (in ? j0 : 0);
         if constexpr (VEC) {
             unsigned* dst = ring + (t & (kAhead - 1)) * 32 * R + lane * NW;
-            if constexpr (C >= 16) {
+            constexpr int VB = C < 16 ? C : 16;
 #pragma unroll
-                for (int q = 0; q < NW; q += 4) copy_async<16>(dst + q, src + (j0 + 4 * q < W ? 4 * q : 0));
-            } else {
-                copy_async<C>(dst, src);
-            }
+            for (int q = 0; q < NW; q += VB / 4)
+                copy_async<VB>(dst + q, src + (j0 + 4 * q < W ? 4 * q : 0), min(max(W - j0 - 4 * q, 0), VB));
         } else {
             unsigned* dst = ring + (t & (kAhead - 1)) * 32 * R + lane * (NW + 1);
-            const unsigned char* word = src - (reinterpret_cast<size_t>(src) & 3);
+            const int off = (int)(reinterpret_cast<size_t>(src) & 3), c = (in ? j0 : 0) - off;
+            const unsigned char* word = src - off;
+            const RowRoom room(inside(u), H, pitch);
 #pragma unroll
-            for (int q = 0; q <= NW; ++q) copy_async<4>(dst + q, word + (word + 4 * q < row + W ? 4 * q : 0), word + 4 * q < row + W);
+            for (int q = 0; q <= NW; ++q) {
+                const bool ok = room.whole(c + 4 * q, W);
+                copy_async<4>(dst + q, word + (ok ? 4 * q : 0), ok ? 4 : 0);
+            }
         }
         copy_commit();
     }
@@ -195,6 +207,11 @@ struct Rows {
 #pragma unroll
         for (int i = 0; i < R; ++i) p[i] = 0u;   // the frame row
         for (int t = 0; t < kAhead; ++t) copy_in(row(t), t);
+        if constexpr (!VEC) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            for (int t = 0; t < min(own, pitch < 3 ? 3 : 1) && in; ++t)
+                first_words(ring + t * 32 * R + lane * (NW + 1), NW, X + (size_t)row(t) * pitch, j0, W, RowRoom(row(t), H, pitch));
+        }
 #pragma unroll 2
         for (int t = 0; t < own; ++t) {
             unsigned on[NW], c[R];

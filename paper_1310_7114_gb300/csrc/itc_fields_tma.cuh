@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(kThreads, (TmaTile<R, ABS, DTYPE, TH, AO, STG,
     __syncthreads();   // s_valid of the first stages
     // (STG) all threads start the copies of the CTA's tile m.  Weights land in place, zeros outside the
     // image.  Byte rows start anywhere: the aligned words that hold a row's bytes are copied as they are
-    // (words without a byte of the row: zeros), and shift_raw moves the bytes into place
+    // (words without a byte of the row or not wholly inside the image: zeros), and shift_raw moves the
+    // bytes into place
     uint32_t* const raw = reinterpret_cast<uint32_t*>(stage0 + STAGE_BYTES);
     auto copy4 = [](void* dst, const void* src, bool ok) {
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
@@ -354,13 +355,15 @@ __global__ void __launch_bounds__(kThreads, (TmaTile<R, ABS, DTYPE, TH, AO, STG,
         if constexpr (DTYPE == ITC_U8) {
             static_assert(TT::RW <= 32, "a lane per raw word of a row");
             const unsigned char* data = reinterpret_cast<const unsigned char*>(d->data);
-#pragma unroll 4
+            const ByteSpan span((long long)(H - 1) * pitch + W);   // (rows above and below the image lie outside it)
+            const int boundary = (int)(reinterpret_cast<uintptr_t>(data + v0) & 3);
+            // (three rows at a time here and all of them in shift_raw: other factors spill 80 bytes at R = 6)
+#pragma unroll 3
             for (int r = tid >> 5; r < ROWS; r += kThreads / 32) {
-                const int u = u0 + r;
-                const unsigned char* row = data + (long long)u * pitch;
-                const unsigned char* word = row + v0 - (reinterpret_cast<uintptr_t>(row + v0) & 3) + 4 * (tid & 31);
-                const bool ok = (unsigned)u < (unsigned)H && word + 3 >= row && word < row + W;
-                if ((tid & 31) < TT::RW) copy4(raw + r * TT::RW + (tid & 31), ok ? word : data - (reinterpret_cast<uintptr_t>(data) & 3), ok);
+                const int u = u0 + r, c = v0 + 4 * (tid & 31) - ((boundary + (u & 3) * (pitch & 3)) & 3);   // the word's first column
+                const long long at = (long long)u * pitch + c;
+                const bool ok = (unsigned)(c + 3) < (unsigned)(W + 3) && span.whole_word(at);
+                if ((tid & 31) < TT::RW) copy4(raw + r * TT::RW + (tid & 31), data + (ok ? at : -(long long)(reinterpret_cast<uintptr_t>(data) & 3)), ok);
             }
         } else {
             const float* data = reinterpret_cast<const float*>(d->data);
@@ -386,12 +389,27 @@ __global__ void __launch_bounds__(kThreads, (TmaTile<R, ABS, DTYPE, TH, AO, STG,
             if ((unsigned)(c + j) < (unsigned)W) keep |= 0xffu << (8 * j);
         const uintptr_t at = reinterpret_cast<uintptr_t>(d->data) + v0 - RA + (long long)(u0 - R) * d->pitch;
         if (q < BW / 4)
-#pragma unroll 4
+#pragma unroll 12
             for (int r = tid >> 5; r < ROWS; r += kThreads / 32) {
                 const int sh = (int)((at + (uintptr_t)r * d->pitch) & 3);
                 reinterpret_cast<uint32_t*>(stage0)[r * (BW / 4) + q] =
                     __funnelshift_r(raw[r * TT::RW + q], raw[r * TT::RW + q + 1], 8 * sh) & keep;
             }
+        // the image's first and last bytes, where their words reach beyond it
+        const int H = d->H, pitch = d->pitch;
+        const uintptr_t first = reinterpret_cast<uintptr_t>(d->data), end = first + (uintptr_t)(H - 1) * pitch + W;
+        auto add_bytes = [&](int u) {   // by the lane that stored the word
+            const int r = u - u0 + R;
+            if (r < 0 || r >= ROWS || (r & (kThreads / 32 - 1)) != tid >> 5 || !keep || q >= BW / 4) return;
+            const uint32_t b = row_bytes(reinterpret_cast<const unsigned char*>(d->data) + (long long)u * pitch, c, W, RowRoom(u, H, pitch));
+            if (b) reinterpret_cast<uint32_t*>(stage0)[r * (BW / 4) + q] |= b;
+        };
+        if (pitch < 3) {   // words span rows
+            for (int u = max(0, u0 - R); u < min(H, u0 - R + ROWS); ++u) add_bytes(u);
+        } else {
+            if (((first | (H == 1 ? end : 0)) & 3) != 0) add_bytes(0);
+            if ((end & 3) != 0 && H > 1) add_bytes(H - 1);
+        }
     };
     if constexpr (STG) copy_tile(0);
     uint32_t phase = 0;   // bit b: parity of the next completion of bar[b]

@@ -311,14 +311,15 @@ __global__ void __launch_bounds__(32 * kRecPairs) rec_cols_scan(const __grid_con
                 hv[q] = f2((float)__ldg(h + o + va), (float)__ldg(h + o + vb));
             }
         };
-        // byte pairs on 2-byte boundaries with one load each (an odd W leaves a padding byte in the
-        // last pair, weighed with 0 below): a warp's load touches 8 image rows whatever it takes from each
+        // byte pairs on 2-byte boundaries with one load each (the last column of an odd W by itself): a
+        // warp's load touches 8 image rows whatever it takes from each
         const unsigned char* hb = reinterpret_cast<const unsigned char*>(D.data);
-        if (D.dtype == ITC_U8 && ((pitch | reinterpret_cast<size_t>(hb)) & 1) == 0) {
+        if (D.dtype == ITC_U8 && ((pitch | reinterpret_cast<size_t>(hb)) & 1) == 0 && W > 1 && (in2 || !in)) {
+            const int at = min(v, (W - 2) & ~1);
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 const size_t o = (size_t)min(32 * (tb + q) + r0, H - 1) * pitch;
-                const uchar2 b = __ldg(reinterpret_cast<const uchar2*>(hb + o + (va & ~1)));
+                const uchar2 b = __ldg(reinterpret_cast<const uchar2*>(hb + o + at));
                 hv[q] = f2((float)b.x, (float)b.y);
             }
         } else if (D.dtype == ITC_U8) {

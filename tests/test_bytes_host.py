@@ -51,3 +51,49 @@ int main() {
 }
 """ % R)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("W,pitch", [(1, 1), (1, 2), (2, 2), (1, 3), (3, 3), (4, 4), (5, 5), (5, 7), (9, 9), (37, 37), (61, 64), (131, 133)])
+def test_row_words(tmp_path, W, pitch):
+    """The words of every row of a byte image on each of the four boundaries, as the kernels take them: whole
+    words inside the image, the bytes that those leave out by themselves; every byte once, and no read
+    outside the image."""
+    r = run_host(tmp_path, """
+int main() {
+    const int W = %d, pitch = %d;
+    alignas(16) unsigned char mem[4096];
+    for (int i = 0; i < 4096; ++i) mem[i] = (unsigned char)(i * 37 + 11) | 1;
+    for (int H = 1; H <= 9; ++H)
+        for (int shift = 0; shift < 4; ++shift) {
+            const unsigned char *data = mem + 64 + shift, *end = data + (H - 1) * pitch + W;
+            for (int u = -9; u < H + 9; ++u) {   // rows above and below the image: nothing
+                const unsigned char* row = data + u * pitch;
+                if (u >= 0 && u < H) continue;
+                for (int c = -((int)((uintptr_t)row & 3)) - 4; c < W; c += 4)
+                    if (c + 3 >= 0 && itc::ByteSpan((H - 1) * pitch + W).whole_word((long long)u * pitch + c)) { printf("row %%d\\n", u); return 1; }
+            }
+            for (int u = 0; u < H; ++u) {
+                const itc::RowRoom room(u, H, pitch);
+                const unsigned char* row = data + u * pitch;
+                const int off = (int)((uintptr_t)row & 3);
+                for (int c = -off - 8; c < W + 12; c += 4) {   // words
+                    const bool whole = room.whole(c, W);
+                    if (whole != (c + 3 >= 0 && c < W && itc::ByteSpan((H - 1) * pitch + W).whole_word((long long)u * pitch + c))) { printf("by offset\\n"); return 1; }
+                    if (whole && (row + c < data || row + c + 4 > end)) { printf("H %%d boundary %%d row %%d word %%d: outside\\n", H, shift, u, c); return 1; }
+                    if (whole && (c + 3 < 0 || c >= W)) { printf("word without a byte of the row\\n"); return 1; }
+                }
+                for (int c = -8; c < W + 12; ++c) {
+                    const uint32_t b = itc::row_bytes(row, c, W, room);
+                    for (int j = 0; j < 4; ++j) {
+                        const int k = c + j;
+                        const bool in = k >= 0 && k < W, whole = room.whole(k - (int)((uintptr_t)(row + k) & 3), W);
+                        const int want = in && !whole ? row[k] : 0;
+                        if ((int)((b >> (8 * j)) & 255) != want) { printf("H %%d boundary %%d row %%d column %%d\\n", H, shift, u, k); return 1; }
+                    }
+                }
+            }
+        }
+    return 0;
+}
+""" % (W, pitch))
+    assert r.returncode == 0, r.stdout + r.stderr
