@@ -168,43 +168,77 @@ __device__ __forceinline__ float moved_to(float w, float delta, int n, bool snap
     return fminf(fmaxf(v, 0.f), (float)(n - 1));
 }
 
-// S_XX of the images of a CTA's group (or of its one image Dg) from their tile partials into
-// s_sxx, one warp per image; gray images (a partial per slice tile) split the kRunThreads / 32 warps
-// evenly over the group's images, eight loads in flight per lane; a fixed order throughout.  Called
+// S_XX of the images of a CTA's group (or of its one image Dg) from their tile partials into s_sxx.
+// A gray image (a partial per slice tile) is always added as four strided shares, a 2-D image as one, in
+// one order whichever warps take them: a warp a share, or where there are as many images as warps an image
+// with its shares side by side (400 images of 64 x 64 x 64: 27 us an evaluation, 29 share by share).  Called
 // by the first kRunThreads threads; s_sxx is valid after the caller's next block barrier.
 template <int ND>
-__device__ __forceinline__ void load_sxx(const RunLaunch& L, const int* grp, int n, const ImageDesc& Dg, double* s_sxx,
-                                         double* s_part, int* s_wpi) {
+constexpr int kSxxShares = ND == 3 ? 4 : 1;
+constexpr int kSxxMost = kGroupMax * kSxxShares<3>;
+template <int ND>
+__device__ __forceinline__ void load_sxx(const RunLaunch& L, const int* grp, int n, const ImageDesc& Dg, double* s_sxx) {
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
-    constexpr int NW = kRunThreads / 32;
-    const int wpi = (ND == 3 && n < NW && !L.sxx_single) ? NW / n : 1;   // warps per image
-    if (tid == 0) *s_wpi = wpi;
+    constexpr int NS = kSxxShares<ND>, NW = kRunThreads / 32;
+    constexpr long long step = 32 * NS;
     if (L.sxx_single) {
-        if (tid == 0) s_sxx[0] = *L.sxx_single;
+        if (tid < NS) s_sxx[tid] = tid == 0 ? *L.sxx_single : 0.0;
         return;
     }
-    for (int g = wid / wpi; g < n; g += NW / wpi) {
-        const ImageDesc& ds = grp ? L.descs[__ldg(grp + 2 + g)] : Dg;
-        const long long nt = ds.sxx_tiles, po = ds.sxx_off, step = 32LL * wpi;
+    auto lane_sum = [&](const double* p, long long nt, int share) {   // eight loads in flight
         double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        long long i = (long long)(wid % wpi) * 32 + lane;
+        long long i = (long long)share * 32 + lane;
         for (; i + 7 * step < nt; i += 8 * step)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] += L.partials[po + i + q * step];
-        for (; i < nt; i += step) v[0] += L.partials[po + i];
-        double t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-        t = warp_sum_d(t);
-        if (lane == 0) {
-            if (wpi == 1) s_sxx[g] = t;
-            else s_part[wid] = t;
+            for (int q = 0; q < 8; ++q) v[q] += p[i + q * step];
+        if (i < nt) {   // the rest, fewer than eight
+            double x[7];
+#pragma unroll
+            for (int q = 0; q < 7; ++q) x[q] = i + q * step < nt ? p[i + q * step] : 0.0;
+#pragma unroll
+            for (int q = 0; q < 7; ++q)
+                if (i + q * step < nt) v[0] += x[q];
         }
+        return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    };
+    const bool images = ND == 3 && n >= NW;
+    for (int g = wid; g < (images ? n : n * NS); g += NW) {
+        const int im = images ? g : g / NS;
+        const ImageDesc& ds = grp ? L.descs[__ldg(grp + 2 + im)] : Dg;
+        const long long nt = ds.sxx_tiles;
+        const double* p = L.partials + ds.sxx_off;
+        if constexpr (ND == 3) {
+            if (images) {
+                double t[NS];
+#pragma unroll
+                for (int q = 0; q < NS; ++q) t[q] = 0;
+                if (nt <= 7 * step) {   // the sums of lane_sum, all shares at once
+#pragma unroll 2
+                    for (long long i = lane; i < nt; i += step)
+#pragma unroll
+                        for (int q = 0; q < NS; ++q) t[q] += i + 32 * q < nt ? p[i + 32 * q] : 0.0;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < NS; ++q) t[q] = lane_sum(p, nt, q);
+                }
+#pragma unroll
+                for (int q = 0; q < NS; ++q) t[q] = warp_sum_d(t[q]);
+                if (lane == 0)
+#pragma unroll
+                    for (int q = 0; q < NS; ++q) s_sxx[g * NS + q] = t[q];
+                continue;
+            }
+        }
+        const double t = warp_sum_d(lane_sum(p, nt, g % NS));
+        if (lane == 0) s_sxx[g] = t;
     }
 }
 // (after the barrier) S_XX of image `sub` of the group
-__device__ __forceinline__ double read_sxx(const double* s_sxx, const double* s_part, int wpi, int sub) {
-    if (wpi == 1) return s_sxx[sub];
+template <int ND>
+__device__ __forceinline__ double read_sxx(const double* s_sxx, int sub) {
     double t = 0;
-    for (int q = 0; q < wpi; ++q) t += s_part[sub * wpi + q];
+#pragma unroll
+    for (int q = 0; q < kSxxShares<ND>; ++q) t += s_sxx[sub * kSxxShares<ND> + q];
     return t;
 }
 
@@ -213,7 +247,7 @@ __device__ __forceinline__ double read_sxx(const double* s_sxx, const double* s_
 // only written after the first of them.
 template <int ND, int SPAN>
 __device__ __forceinline__ void iterate_group(const RunLaunch& L, const int* grp, int n, float* s_pos, float2* s_red,
-                                              int* s_mv, const double* s_sxx, const double* s_part, int wpi) {
+                                              int* s_mv, const double* s_sxx) {
     constexpr int WPI = SPAN / 32;   // warps per image (0: two images per warp)
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int sub = tid / SPAN, kl = tid % SPAN;
@@ -310,7 +344,7 @@ __device__ __forceinline__ void iterate_group(const RunLaunch& L, const int* grp
         }
         if (!L.final_eval && t == 0 && L.stats && (SPAN <= 32 || kl < 32))
             write_stats(L.stats + (has ? img : 0), has && kl == 0, SPAN == 16 ? (lane & 16) : 0, s,
-                        read_sxx(s_sxx, s_part, wpi, has ? sub : 0), 0, 0, Dg.dcs_const,
+                        read_sxx<ND>(s_sxx, has ? sub : 0), 0, 0, Dg.dcs_const,
                         has && L.img_status ? L.img_status[img] : ITC_OK);
         if (!upd) live = false;
         // threads that do not update divide 1 by 1 (0 / 0 would take the slow division path and
@@ -352,7 +386,7 @@ __device__ __forceinline__ void iterate_group(const RunLaunch& L, const int* grp
     }
     if (L.stats && L.final_eval && (SPAN <= 32 || kl < 32))
         write_stats(L.stats + (has ? img : 0), has && kl == 0, SPAN == 16 ? (lane & 16) : 0, s,
-                    read_sxx(s_sxx, s_part, wpi, has ? sub : 0), moved, done, Dg.dcs_const,
+                    read_sxx<ND>(s_sxx, has ? sub : 0), moved, done, Dg.dcs_const,
                     has && L.img_status ? L.img_status[img] : ITC_OK);
     if (has && !L.final_eval && L.stats && kl == 0) {
         L.stats[img].moved = moved;
@@ -375,7 +409,7 @@ __device__ __forceinline__ void iterate_group(const RunLaunch& L, const int* grp
 // barrier and the pair loop ran one step at a time).
 template <int ND>
 __device__ __forceinline__ void iterate_wide(const RunLaunch& L, int img, const ImageDesc& Dg, float* pos, float4* s_half,
-                                             float2* s_red, int* s_mv, const double* s_sxx, const double* s_part, int wpi) {
+                                             float2* s_red, int* s_mv, const double* s_sxx) {
     constexpr int SPAN = kRunThreads / 2;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int kl = tid % SPAN;
@@ -456,7 +490,7 @@ __device__ __forceinline__ void iterate_wide(const RunLaunch& L, int img, const 
             s.sww = y;
             if (last) s.empty = s_mv[0] + s_mv[1];
             if (!L.final_eval && t == 0 && L.stats && kl < 32)
-                write_stats(L.stats + img, kl == 0, 0, s, read_sxx(s_sxx, s_part, wpi, 0), 0, 0, Dg.dcs_const,
+                write_stats(L.stats + img, kl == 0, 0, s, read_sxx<ND>(s_sxx, 0), 0, 0, Dg.dcs_const,
                             L.img_status ? L.img_status[img] : ITC_OK);
             if (upd) {
                 const float c = x / y;
@@ -487,7 +521,7 @@ __device__ __forceinline__ void iterate_wide(const RunLaunch& L, int img, const 
     }
     if (!owner) return;
     if (L.stats && L.final_eval && kl < 32)
-        write_stats(L.stats + img, kl == 0, 0, s, read_sxx(s_sxx, s_part, wpi, 0), moved, done, Dg.dcs_const,
+        write_stats(L.stats + img, kl == 0, 0, s, read_sxx<ND>(s_sxx, 0), moved, done, Dg.dcs_const,
                     L.img_status ? L.img_status[img] : ITC_OK);
     if (!L.final_eval && L.stats && kl == 0) {
         L.stats[img].moved = moved;
@@ -560,16 +594,16 @@ __device__ __forceinline__ void iterate_large(const RunLaunch& L) {
     float2* as = reinterpret_cast<float2*>(posz + (ND == 3 ? mp : 0));   // (a_k, s_k) of every vector
     float* st = reinterpret_cast<float*>(as + mp);   // this CTA's vectors: planes of `share` floats:
     // even s, even E[ND], odd s, odd E[ND], a, D[ND]
-    __shared__ double s_sxx[kGroupMax], s_part[kRunThreads / 32];
+    __shared__ double s_sxx[kSxxMost];
     __shared__ float2 s_red[kRunThreads / 32];
-    __shared__ int s_wpi, s_empty, s_mv, s_cnt[kLargeCluster];   // s_cnt: moved vectors of every CTA
+    __shared__ int s_empty, s_mv, s_cnt[kLargeCluster];   // s_cnt: moved vectors of every CTA
     const float* Win = L.W_in + Dg.w_off;
     for (int k = tid; k < mp; k += NT) {
         pos[large_at<SPLIT>(k)] = k < M ? Win[k * ND] : kFar;
         pos[large_at<SPLIT>(k) + 2] = k < M ? Win[k * ND + 1] : kFar;
         if constexpr (ND == 3) posz[large_atz<SPLIT>(k)] = k < M ? Win[k * ND + 2] : kFar;
     }
-    if (tid < kRunThreads) load_sxx<ND>(L, grp, 1, Dg, s_sxx, s_part, &s_wpi);
+    if (tid < kRunThreads) load_sxx<ND>(L, grp, 1, Dg, s_sxx);
     auto load_w = [&](int k, float (&w)[ND]) {
         w[0] = pos[large_at<SPLIT>(k)];
         w[1] = pos[large_at<SPLIT>(k) + 2];
@@ -649,7 +683,7 @@ __device__ __forceinline__ void iterate_large(const RunLaunch& L) {
             __syncthreads();
             s.empty = s_empty;
             if (rank == 0 && wid == 0)
-                write_stats(L.stats + img, lane == 0, 0, s, read_sxx(s_sxx, s_part, s_wpi, 0), 0, 0, Dg.dcs_const,
+                write_stats(L.stats + img, lane == 0, 0, s, read_sxx<ND>(s_sxx, 0), 0, 0, Dg.dcs_const,
                             L.img_status ? L.img_status[img] : ITC_OK);
         }
         if (t == D.iters || stop) break;   // uniform over the cluster
@@ -700,7 +734,7 @@ __device__ __forceinline__ void iterate_large(const RunLaunch& L) {
     __syncthreads();
     if (rank == 0 && L.stats && L.final_eval && wid == 0) {
         s.empty = s_empty;
-        write_stats(L.stats + img, lane == 0, 0, s, read_sxx(s_sxx, s_part, s_wpi, 0), moved, done, Dg.dcs_const,
+        write_stats(L.stats + img, lane == 0, 0, s, read_sxx<ND>(s_sxx, 0), moved, done, Dg.dcs_const,
                     L.img_status ? L.img_status[img] : ITC_OK);
     }
     if (rank == 0 && L.stats && !L.final_eval && tid == 0) {
@@ -726,7 +760,6 @@ __global__ void __launch_bounds__(large_threads(SPLIT), SPLIT ? 1 : (ND == 3 ? 6
 }
 
 // ND: lattice dimension (2 or 3).
-// ND: lattice dimension (2 or 3).
 // Register budget: 7 CTAs per SM in 2-D and 6 in 3-D leave the per-iteration state in registers
 // (8 CTAs per SM spilled it and lengthened every iteration).
 template <int ND>
@@ -746,19 +779,15 @@ __global__ void __launch_bounds__(kRunThreads, ND == 3 ? 6 : 7) run_kernel(const
     __shared__ __align__(16) float2 s_red[kRunThreads / 32];
     __shared__ float4 s_half[kRunThreads / 2];
     __shared__ int s_mv[kRunThreads / 32];
-    __shared__ double s_sxx[kGroupMax];
-    __shared__ double s_part[kRunThreads / 32];   // S_XX partial sums of the warps
-    __shared__ int s_wpi;
-    load_sxx<ND>(L, grp, n, Dg, s_sxx, s_part, &s_wpi);
+    __shared__ double s_sxx[kSxxMost];
+    load_sxx<ND>(L, grp, n, Dg, s_sxx);
     __syncthreads();
-    const int wpi = s_wpi;
-    if (span == 16) iterate_group<ND, 16>(L, grp, n, s_pos, s_red, s_mv, s_sxx, s_part, wpi);
-    else if (span == 32) iterate_group<ND, 32>(L, grp, n, s_pos, s_red, s_mv, s_sxx, s_part, wpi);
+    if (span == 16) iterate_group<ND, 16>(L, grp, n, s_pos, s_red, s_mv, s_sxx);
+    else if (span == 32) iterate_group<ND, 32>(L, grp, n, s_pos, s_red, s_mv, s_sxx);
     else if (span == 64 && n == 1)
-        iterate_wide<ND>(L, grp ? __ldg(grp + 2) : L.img_base + (int)blockIdx.x, Dg, s_pos, s_half, s_red, s_mv, s_sxx,
-                         s_part, wpi);
-    else if (span == 64) iterate_group<ND, 64>(L, grp, n, s_pos, s_red, s_mv, s_sxx, s_part, wpi);
-    else iterate_group<ND, 128>(L, grp, n, s_pos, s_red, s_mv, s_sxx, s_part, wpi);
+        iterate_wide<ND>(L, grp ? __ldg(grp + 2) : L.img_base + (int)blockIdx.x, Dg, s_pos, s_half, s_red, s_mv, s_sxx);
+    else if (span == 64) iterate_group<ND, 64>(L, grp, n, s_pos, s_red, s_mv, s_sxx);
+    else iterate_group<ND, 128>(L, grp, n, s_pos, s_red, s_mv, s_sxx);
 }
 
 // CTAs per image of a launch with nlarge images of more than kRunThreads vectors: as many as give
