@@ -271,6 +271,12 @@ struct Rows {
     }
 };
 
+// An image of one column: the frame lies beside every pixel (the walks' pairs would take two columns of the row)
+__device__ __noinline__ void one_column(const ImageDesc& D, float* out) {
+    const unsigned char* X = reinterpret_cast<const unsigned char*>(D.data);
+    for (int u = threadIdx.x; u < D.H; u += blockDim.x) out[D.pad_off + (size_t)u * D.fpitch] = X[(size_t)u * D.pitch] ? 3.f : 0.f;
+}
+
 template <int C>
 __device__ __forceinline__ void run_rows(const ImageDesc& D, float* out, unsigned* ring) {
     constexpr int VB = C < 16 ? C : 16;   // bytes per vector load
@@ -285,7 +291,8 @@ __global__ void __launch_bounds__(64) chamfer_kernel(const __grid_constant__ Cha
     const int W = D.W;
     __shared__ __align__(16) unsigned rings[2][kAhead * 32 * (CMAX / 2)];
     unsigned* ring = rings[threadIdx.x >> 5];
-    if (W <= 128) run_rows<4>(D, L.out, ring);
+    if (W == 1) one_column(D, L.out);
+    else if (W <= 128) run_rows<4>(D, L.out, ring);
     else if (W <= 256) { if constexpr (CMAX >= 8) run_rows<8>(D, L.out, ring); }
     else if (W <= 512) { if constexpr (CMAX >= 16) run_rows<16>(D, L.out, ring); }
     else { if constexpr (CMAX >= 32) run_rows<32>(D, L.out, ring); }
