@@ -342,8 +342,8 @@ class Plan:
         self._keep = (images, weights)
 
     @property
-    def host_ptr(self) -> int:
-        return ctypes.addressof(self.host)
+    def host_ptr(self):
+        return _P(ctypes.addressof(self.host))
 
     def budget_bytes(self, budget_bytes: int = 0) -> int:
         """itc_plan_budget_bytes: workspace of the budgeted calls within ``budget_bytes`` in all
