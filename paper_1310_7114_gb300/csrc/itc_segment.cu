@@ -13,7 +13,7 @@
 // and 16 x 16 tiles without data only write -1.  For the others the codebooks that can win somewhere
 // are listed, first for the block and from that list for each tile: with dmin_k / dmax_k the metric
 // of the nearest / farthest point of the box, every k with dmin_k <= min_j dmax_j (the same rounded
-// arithmetic, which is monotone in each |d_i|, so the bounds hold for every pixel).  Lists keep k
+// arithmetic, which is monotone in each |d_i|, so the bounds hold for every pixel; a list is never empty).  Lists keep k
 // order, so the first strict minimum over one is the lowest index on ties.  A lane then takes 8 rows
 // of one column: the column's term once per codebook, the rows' terms and sums as packed operations.
 // Bound by instruction issue (the bytes take 38 us).  1024 ragged shapes (64 to 512 px a side, M 16 to
@@ -74,8 +74,10 @@ __device__ __forceinline__ int list_box(const SegSmem& S, const unsigned short* 
         if (i < n) {
             k = from ? from[i] : i;
             const float2 r = S.site[k];
-            hit = __fadd_rn(term(fmaxf(fmaxf(fu0 - r.x, r.x - fu1), 0.f), q[0]),
-                            term(fmaxf(fmaxf(fv0 - r.y, r.y - fv1), 0.f), q[1])) <= bound;
+            // (not greater, so that a NaN, an infinite q times 0, stays: at such widths all metrics are
+            // infinite or NaN, no comparison holds and the first vector keeps every pixel)
+            hit = !(__fadd_rn(term(fmaxf(fmaxf(fu0 - r.x, r.x - fu1), 0.f), q[0]),
+                              term(fmaxf(fmaxf(fv0 - r.y, r.y - fv1), 0.f), q[1])) > bound);
         }
         const unsigned bal = __ballot_sync(kFull, hit);
         if (hit) to[nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)k;
