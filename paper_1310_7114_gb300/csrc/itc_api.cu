@@ -157,10 +157,6 @@ void fill_desc(const itc_image* img, const itc_params* p, int M, ImageDesc* d) {
     const int th = tile_h_of(img->ndim);
     d->tiles_u = (img->H + th - 1) / th;
     d->tiles_v = (img->W + kTileW - 1) / kTileW;
-    if (p->flags & ITC_RECURSIVE) {   // one S_XX partial per 8 (long sides: 32) columns
-        d->tiles_u = 1;
-        d->tiles_v = rec_scans(img->H, img->W) ? (img->W + 7) / 8 : (img->W + 31) / 32;
-    }
     d->tiles_g = img->ndim == 3 ? d->G : 1;   // 3-D tiles: one gray slice each
     d->plane_floats = (long long)d->G * img->H * d->fpitch;
     d->bwd_tiles_u = (img->H + kBwdTileH - 1) / kBwdTileH;
@@ -203,8 +199,9 @@ size_t plan_layout(int B, size_t* desc_off, size_t* ints_off, size_t* tmap_off =
     const size_t h = align_up(sizeof(PlanHeader), 256);
     const size_t d = align_up((size_t)B * sizeof(ImageDesc), 256);
     // per class an image list and a tile prefix (an image is in at most two classes: its
-    // fields class and its self-overlap class), then the backward image order
-    const size_t n = align_up((size_t)((5 + kGroupInts) * (size_t)B + kMaxClasses + 2) * sizeof(int), 256);
+    // fields class and its self-overlap class), then the backward image order, the iteration groups and
+    // two lists per class of recursive images
+    const size_t n = align_up((size_t)((9 + kGroupInts) * (size_t)B + kMaxClasses + 2) * sizeof(int), 256);
     const size_t m = align_up((size_t)2 * B * sizeof(CUtensorMap), 256);   // fields pass, self-overlap pass
     if (desc_off) *desc_off = h;
     if (ints_off) *ints_off = h + d;
@@ -326,6 +323,125 @@ int lower_pos(const int* list, int n, int b) {
         if (list[mid] < b) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// Which images of a recursive class are filtered sequentially: those with a side of more than kRecMaxLine,
+// and where that is faster those with no side above the returned one.  Scans cost a line's time whatever its
+// length; sequential recursions cost a sample's, once the batch has lines enough to fill the GPU, and one
+// chain of samples at least.  Fitted to 102 batches of 0.25 to 48 Mpx of images of 32 to 1024 px (microseconds,
+// W samples a row): a scanned row (1 + W / 256) / 1000, more where long lines leave few CTAs on an SM, 28 in all
+// at least; sequential 1/48 per 1000 samples in whole warps of 32 lines, the longer of that and the chain with
+// 0.3 of the other, or with all of it beside the chain of a long image.  The choice is the better one or within
+// 10 % of it in 101 of them (48 Mpx of 48 to 192 px: 12 %).  16 Mpx of 32, 64, 96, 128, 192 and 512 px: scans
+// 1149, 628, 472, 379, 311, 261, sequential 410, 330, 313, 335, 395, 557.
+int rec_seq_side(const ClassInfo& ci, const ImageDesc* descs, const int* list) {
+    auto few = [](double n) { return n <= 256 ? 1.0 : (n <= 512 ? 1.25 : (n <= 1024 ? 1.8 : 2.9)); };
+    bool longer = false;
+    auto cost = [&](int side) {
+        double chain = 0, samples = 0, scan = 0;
+        for (int i = 0; i < ci.nimg; ++i) {
+            const ImageDesc& d = descs[list[i]];
+            const double H = d.H, W = d.W;
+            const bool scans = rec_scans(d.H, d.W);
+            if (scans && std::max(d.H, d.W) > side) {
+                scan += H * (1 + W / 256) * few(W) + W * (1 + H / 256) * few(H);
+                continue;
+            }
+            longer |= !scans;
+            chain = std::max(chain, 20 + 0.23 * W + 0.35 * H);
+            samples += 0.5 * ((double)align_up(d.H, 32) * W + (double)align_up(d.W, 32) * H);
+        }
+        samples /= 48e3;
+        return std::max(chain, samples) + (longer ? 1.0 : 0.3) * std::min(chain, samples) + (scan > 0 ? 28 + scan / 1000 : 0);
+    };
+    int best = 0;
+    double least = cost(0);
+    if (!longer) least *= 0.92;   // (the scans are the more accurate: 1.6e-6 of the field, 3.3e-6)
+    for (int side : {64, 96, 128, 192, 256}) {
+        const double t = cost(side);
+        if (t < least) {
+            least = t;
+            best = side;
+        }
+    }
+    return best;
+}
+
+// The launches of a recursive class's scans, per axis.  A launch's shared memory follows its longest line
+// (201 KB for 2048 samples, one CTA of 8 lines per SM; 28 KB for 256) and its grid the image with the most
+// lines, so images with shorter lines (up to 256, 512, 1024 samples) or fewer lines (the same steps) have a
+// launch of their own where that is worth the time of one: four times as many CTAs per SM and more of them
+// than the longer lines' launch takes in four waves (152 SMs), or 50 000 CTAs without lines left out.
+// Microseconds with all images in one launch and now: 256 of 128 x 128 with one of 2048 x 2048 937 and 249
+// (sequential 1926), 47 of 500 x 500 with the same 595 and 352 (2165), 300 of 100 x 100 with 20 of 600 x 600 297
+// and 242 (655); 48 of 128 to 1024 px, in one launch, 555.  Splitting at twice the CTAs per SM made those 575.
+void rec_groups(ClassInfo& ci, const ImageDesc* descs, int* ints, int& io) {
+    const int* list = ints + ci.list_off;
+    const int arrays = ci.self ? 2 : 3;
+    auto step_of = [](int n) { return n <= 256 ? 0 : (n <= 512 ? 1 : (n <= 1024 ? 2 : 3)); };
+    auto ctas_per_sm = [&](int len) { return std::min(16, (int)(227 * 1024 / (rec_smem_bytes(len, arrays) + 1024))); };
+    auto blocks_of = [](int lines) { return (lines + kRecLines - 1) / kRecLines; };
+    for (int axis = 0; axis < 2; ++axis) {
+        struct Cell { long long blocks; int n, len, lines, group; } cell[4][4] = {};   // by line length, by lines
+        auto cell_of = [&](const ImageDesc& d) -> Cell* {
+            if (d.rec_seq) return nullptr;
+            return &cell[step_of(axis ? d.W : d.H)][step_of(axis ? d.H : d.W)];
+        };
+        for (int i = 0; i < ci.nimg; ++i) {
+            const ImageDesc& d = descs[list[i]];
+            Cell* c = cell_of(d);
+            if (!c) continue;
+            c->len = std::max(c->len, axis ? d.W : d.H);
+            c->lines = std::max(c->lines, axis ? d.H : d.W);
+            c->blocks += blocks_of(axis ? d.H : d.W);
+            ++c->n;
+        }
+        int ng = 0;
+        RecGroup* G = ci.rec_scan[axis];
+        bool open = false;
+        for (int k = 3; k >= 0; --k) {   // the longest lines first
+            long long blocks = 0;
+            int len = 0, n = 0;
+            for (const Cell& c : cell[k]) {
+                blocks += c.blocks;
+                len = std::max(len, c.len);
+                n += c.n;
+            }
+            if (n == 0) continue;
+            if (open && ctas_per_sm(len) >= 4 * ctas_per_sm(G[ng - 1].len) &&
+                blocks > 4LL * kSoloImages * ctas_per_sm(G[ng - 1].len))
+                open = false;
+            for (int l = 3; l >= 0; --l) {   // the most lines first
+                Cell& c = cell[k][l];
+                if (c.n == 0) continue;
+                if (!open || (long long)c.n * blocks_of(G[ng - 1].lines) - c.blocks > 50000) {
+                    G[ng++] = {0, 0, 0, 0};
+                    open = true;
+                }
+                c.group = ng - 1;
+                G[ng - 1].len = std::max(G[ng - 1].len, c.len);
+                G[ng - 1].lines = std::max(G[ng - 1].lines, c.lines);
+            }
+        }
+        ci.rec_ngroups[axis] = ng;
+        for (int g = 0; g < ng; ++g) {
+            G[g].off = io;
+            for (int i = 0; i < ci.nimg; ++i) {
+                const Cell* c = cell_of(descs[list[i]]);
+                if (c && c->group == g) ints[io++] = list[i];
+            }
+            G[g].n = io - G[g].off;
+        }
+    }
+    ci.rec_seq = {io, 0, 0, 0};
+    for (int i = 0; i < ci.nimg; ++i) {
+        const ImageDesc& d = descs[list[i]];
+        if (!d.rec_seq) continue;
+        ints[io++] = list[i];
+        ++ci.rec_seq.n;
+        ci.rec_seq.len = std::max(ci.rec_seq.len, d.W);
+        ci.rec_seq.lines = std::max(ci.rec_seq.lines, d.H);
+    }
 }
 
 const PlanHeader* plan_of(const void* plan_host) {
@@ -608,6 +724,19 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         ci.prefix_off = io;
         io += n + 1;
     }
+    // recursive fields: how each image's lines are filtered; one S_XX partial per 8 (sequential: 32) columns
+    for (int c = 0; c < h->ncls; ++c) {
+        const ClassInfo& ci = h->cls[c];
+        if (!ci.recursive || ci.self) continue;
+        const int side = rec_seq_side(ci, descs, ints + ci.list_off);
+        for (int i = 0; i < ci.nimg; ++i) {
+            ImageDesc& d = descs[ints[ci.list_off + i]];
+            d.rec_seq = !rec_scans(d.H, d.W) || std::max(d.H, d.W) <= side;
+            d.tiles_u = 1;
+            d.tiles_v = d.rec_seq ? (d.W + 31) / 32 : (d.W + kRecLines - 1) / kRecLines;
+            d.self_tiles_u = d.tiles_u;
+        }
+    }
     // S_XX partials: room for the most tiles any tunable tile height can give (32-row tiles)
     long long pcap = 0;
     {
@@ -669,6 +798,9 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         h->run_nlarge[nd - 2] = nl;
         h->run_ngroups[nd - 2] = ng - nl;
     }
+    const int count_ints = io;
+    for (int c = 0; c < h->ncls; ++c)
+        if (h->cls[c].recursive) rec_groups(h->cls[c], descs, ints, io);
     h->nints = io;
     h->bwd_order_off = bwd_off;
     h->run_groups_off = run_off;
@@ -686,7 +818,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
     h->ws_status_off = (long long)off;
     off = align_up(off + (size_t)B * sizeof(int), 256);
     h->ws_count_off = (long long)off;
-    off = align_up(off + (size_t)io * sizeof(int), 256);   // io: every class list position fits
+    off = align_up(off + (size_t)count_ints * sizeof(int), 256);   // every class list position fits
     h->ws_bytes = (long long)off;
     if (ws_bytes_out) *ws_bytes_out = off;
     memcpy(plan, buf.data(), need);
@@ -760,10 +892,21 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
             R.descs = L.descs;
             R.fields = L.fields;
             R.partials = L.partials;
-            R.img_list = L.img_list;
-            R.pos_base = p0;
             R.mode = L.mode;
-            rc = cuda_status(launch_recursive(R, p1 - p0, h->max_dim[0], h->max_dim[1], s));
+            // the images of the range in a group's list
+            auto images = [&](const RecGroup& g) {
+                const int q0 = lower_pos(hints + g.off, g.n, b0), q1 = lower_pos(hints + g.off, g.n, b1);
+                R.img_list = ints + g.off + q0;
+                return q1 - q0;
+            };
+            int n = images(ci.rec_seq);
+            rc = cuda_status(launch_recursive_seq(R, n, ci.rec_seq.lines, ci.rec_seq.len, s));
+            for (int axis = 1; axis >= 0; --axis)
+                for (int g = 0; g < ci.rec_ngroups[axis] && !rc; ++g) {
+                    const RecGroup& G = ci.rec_scan[axis][g];
+                    n = images(G);
+                    rc = cuda_status(launch_recursive_scan(R, axis, n, G.lines, G.len, s));
+                }
         } else {
             rc = cuda_status(launch_fields_any(L, ci.tma != 0 && !ci.use_plain, t0, t1, ci.taps.R[0],
                                                ci.taps.R[1], ci.ndim, ci.dtype, s));

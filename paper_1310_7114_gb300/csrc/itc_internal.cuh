@@ -45,10 +45,23 @@ struct RecCoef {
     float pr[2][2][5], pi[2][2][5];   // z^(seg 2^k), seg = ceil(side / 32): a lane's share of a line
 };
 
-// Recursive fields of images with no side longer than this filter each line with a warp in shared
+// Recursive fields of images with no side longer than this can filter each line with a warp in shared
 // memory (three arrays of 8 lines: 201 KB); others run one sequential recursion per line.
 constexpr int kRecMaxLine = 2048;
 __host__ __device__ constexpr bool rec_scans(int H, int W) { return H <= kRecMaxLine && W <= kRecMaxLine; }
+constexpr int kRecPairs = 4;               // line pairs (warps) per CTA of the scan kernels
+constexpr int kRecLines = 2 * kRecPairs;
+// Shared float2's of a pair of lines of n samples with `arrays` arrays; 4 more than a multiple of 32,
+// so that the 4 column pairs x 8 rows a warp stages at a time spread over the banks.
+__host__ __device__ constexpr int rec_pair_floats2(int n, int arrays) { return arrays * 32 * (((n + 31) / 32) | 1) + 4; }
+__host__ __device__ constexpr size_t rec_smem_bytes(int n, int arrays) { return (size_t)kRecPairs * rec_pair_floats2(n, arrays) * 8; }
+
+// Images of a recursive class that share a launch: n entries from `off` of the plan's int area on, ascending;
+// their longest line and the most lines of one of them (sequential: the largest W and H).
+struct RecGroup {
+    int off, n, len, lines;
+};
+constexpr int kRecGroups = 16;             // most per axis: four steps of line length, four of the number of lines
 
 // One image as the kernels see it (device-resident inside a plan, or passed by value).
 struct ImageDesc {
@@ -84,6 +97,7 @@ struct ImageDesc {
     long long pad_off;          // offset (floats) of the image in the padded per-pixel layout
                                 // (H rows of fpitch floats; chamfer weights)
     RecCoef rc, rc_self;        // ITC_RECURSIVE: the recursions at sigma and at the V(X) width
+    int rec_seq;                // its lines are filtered one sample after another, not by scans
 };
 
 
@@ -97,6 +111,8 @@ struct ClassInfo {
     float tuned_ms;             // fields time of the class under the chosen configuration (0: untuned)
     int self;                   // self-overlap class: A at width s only, plain tiles
     int recursive;              // fields by recursive filtering (ITC_RECURSIVE); widths per image
+    RecGroup rec_scan[2][kRecGroups], rec_seq;   // its scanned images by line length along u and along v, and
+    int rec_ngroups[2];                          // those filtered sequentially
     int list_off;               // offset (ints) of this class's image list in the plan int area
     int prefix_off;             // offset (ints) of the class tile prefix (nimg + 1 ints)
     long long partial_base;     // first partial of the class
@@ -250,8 +266,7 @@ struct RecursiveLaunch {
     const ImageDesc* descs;
     float* fields;              // fields base (the images' planes and scratch planes)
     double* partials;
-    const int* img_list;        // class image list
-    int pos_base;               // first list position of this launch
+    const int* img_list;        // images of this launch
     int mode;                   // 0: A, F_u, F_v and S_XX; 1: A_s and S_XX (self-overlap pass)
 };
 
@@ -308,7 +323,11 @@ cudaError_t launch_fields_tma_self_f32(const FieldsLaunch& L, int ntiles, int R,
 // of the others; else both are the range's image count.  work: most (iters + 1) M^2 of a large image.
 cudaError_t launch_run(const RunLaunch& L, int large_ctas, int nlarge, int ctas, int max_M, double work, cudaStream_t s,
                        int ndim);
-cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
+// nimg images of L.img_list with lines of up to `len` samples along v (axis 1) or u (axis 0), at most
+// `lines` of them each; axis 1 of every image before axis 0 of any
+cudaError_t launch_recursive_scan(const RecursiveLaunch& L, int axis, int nimg, int lines, int len, cudaStream_t s);
+// both axes of images whose lines are filtered sequentially
+cudaError_t launch_recursive_seq(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
 cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
 // max_blocks: most 64 x 64 pixel blocks of one image; kinds: bit kSeg* for each kind of image in the plan
 cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int kinds, cudaStream_t s);

@@ -26,7 +26,8 @@
 // 48 images of 128 to 1024 px a side (15 Mpx), microseconds, before and now: along v 431 and 102, along u
 // 694 and 245, the self-overlap pass 361 and 60, 567 and 105.
 //
-// Longer lines keep one sequential recursion per row and column (rec_rows_kernel, rec_cols_kernel):
+// Longer lines, and small images where a batch has lines enough to fill the GPU (rec_seq_side in itc_api.cu),
+// take one sequential recursion per row and column (rec_rows_kernel, rec_cols_kernel):
 // along v one lane per row, rows staged through shared memory in 32 x 32 tiles, the causal part
 // stored and the anticausal part added; along u one thread per column, 128 columns per CTA, rows in
 // prefetched chunks, one S_XX partial per 32 columns.
@@ -43,10 +44,9 @@ __device__ __forceinline__ Cplx cmul(Cplx a, Cplx b) { return {a.r * b.r - a.i *
 __device__ __forceinline__ Cplx cadd(Cplx a, Cplx b) { return {a.r + b.r, a.i + b.i}; }
 __device__ __forceinline__ float re_mul(Cplx c, Cplx s) { return c.r * s.r - c.i * s.i; }
 
-// the image of the CTA: the class list entry of position base + blockIdx.x (blockIdx.y picks the
-// CTA's block of rows or columns within it)
+// the image of the CTA: list entry blockIdx.x (blockIdx.y picks the CTA's block of rows or columns within it)
 __device__ __forceinline__ const ImageDesc& rec_image(const RecursiveLaunch& L) {
-    return L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x)];
+    return L.descs[__ldg(L.img_list + blockIdx.x)];
 }
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
@@ -72,9 +72,6 @@ template <bool UP>
 __device__ __forceinline__ Cplx2 shfl_by(const Cplx2& s, int o) {
     return {f2(shfl_by<UP>(s.r.x, o), shfl_by<UP>(s.r.y, o)), f2(shfl_by<UP>(s.i.x, o), shfl_by<UP>(s.i.y, o))};
 }
-
-constexpr int kRecPairs = 4;               // line pairs (warps) per CTA of the scan kernels
-constexpr int kRecLines = 2 * kRecPairs;
 
 // One axis of the recursion: z, the weights and z^(seg 2^k) of both terms.
 struct RecAxis {
@@ -205,16 +202,12 @@ struct LineAt {
     }
 };
 
-// Shared float2's of a pair of lines of n samples with `arrays` arrays; 4 more than a multiple of 32,
-// so that the 4 column pairs x 8 rows a warp stages at a time spread over the banks.
-__host__ __device__ constexpr int rec_pair_floats2(int n, int arrays) { return arrays * 32 * (((n + 31) / 32) | 1) + 4; }
-
 template <bool MOM>
 __global__ void __launch_bounds__(32 * kRecPairs) rec_rows_scan(const __grid_constant__ RecursiveLaunch L, int nblk) {
-    const ImageDesc& D = L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x / nblk)];
+    const ImageDesc& D = L.descs[__ldg(L.img_list + blockIdx.x / nblk)];
     const int H = D.H, W = D.W, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int u = (blockIdx.x % nblk) * kRecLines + 2 * wid;
-    if (!rec_scans(H, W) || u >= H) return;   // no block-wide barrier below
+    if (u >= H) return;   // no block-wide barrier below
     const int seg = (W + 31) / 32, str = seg | 1;
     const bool two = u + 1 < H;
     const RecAxis ax(MOM ? D.rc : D.rc_self, 1);
@@ -272,10 +265,10 @@ __global__ void __launch_bounds__(32 * kRecPairs) rec_rows_scan(const __grid_con
 template <int PART>
 __global__ void __launch_bounds__(32 * kRecPairs) rec_cols_scan(const __grid_constant__ RecursiveLaunch L, int nblk) {
     constexpr bool MOM = PART == 0;
-    const ImageDesc& D = L.descs[__ldg(L.img_list + L.pos_base + blockIdx.x / nblk)];
+    const ImageDesc& D = L.descs[__ldg(L.img_list + blockIdx.x / nblk)];
     const int H = D.H, W = D.W, fp = D.fpitch, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int blk = blockIdx.x % nblk, v0 = blk * kRecLines;
-    if (!rec_scans(H, W) || v0 >= W) return;
+    if (v0 >= W) return;
     const int seg = (H + 31) / 32, str = seg | 1, ls = rec_pair_floats2(H, MOM ? 3 : 2);
     extern __shared__ __align__(16) float2 rsm2[];
     __shared__ double red[kRecPairs];
@@ -311,11 +304,11 @@ __global__ void __launch_bounds__(32 * kRecPairs) rec_cols_scan(const __grid_con
                 hv[q] = f2((float)__ldg(h + o + va), (float)__ldg(h + o + vb));
             }
         };
-        // byte pairs on 2-byte boundaries with one load each (the last column of an odd W by itself): a
-        // warp's load touches 8 image rows whatever it takes from each
+        // byte pairs on 2-byte boundaries with one load each (not in the CTA that holds the last column of an
+        // odd W): a warp's load touches 8 image rows whatever it takes from each
         const unsigned char* hb = reinterpret_cast<const unsigned char*>(D.data);
-        if (D.dtype == ITC_U8 && ((pitch | reinterpret_cast<size_t>(hb)) & 1) == 0 && W > 1 && (in2 || !in)) {
-            const int at = min(v, (W - 2) & ~1);
+        if (D.dtype == ITC_U8 && ((pitch | reinterpret_cast<size_t>(hb)) & 1) == 0 && ((W & 1) == 0 || v0 + kRecLines <= W)) {
+            const int at = min(v, W - 2);
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 const size_t o = (size_t)min(32 * (tb + q) + r0, H - 1) * pitch;
@@ -390,7 +383,6 @@ template <bool MOM>   // MOM: the moment fields too (else the self-overlap pass:
 __global__ void __launch_bounds__(32 * kRecRowWarps) rec_rows_kernel(const __grid_constant__ RecursiveLaunch L) {
     const ImageDesc& D = rec_image(L);
     const int H = D.H, W = D.W, fp = D.fpitch, pitch = D.pitch;
-    if (rec_scans(H, W)) return;
     float* P0 = L.fields + (MOM ? D.field_off + 3 * D.plane_floats : D.self_off + D.plane_floats);
     float* P1 = P0 + D.plane_floats;   // T_v (moments only)
     const RecCoef& rc = MOM ? D.rc : D.rc_self;
@@ -505,7 +497,6 @@ template <bool MOM>
 __global__ void __launch_bounds__(kRecColThreads) rec_cols_kernel(const __grid_constant__ RecursiveLaunch L) {
     const ImageDesc& D = rec_image(L);
     const int H = D.H, W = D.W, fp = D.fpitch;
-    if (rec_scans(H, W)) return;
     const long long pl = D.plane_floats;
     const float* T = L.fields + (MOM ? D.field_off + 3 * pl : D.self_off + pl);
     const float* Tv = T + pl;
@@ -612,33 +603,24 @@ __global__ void __launch_bounds__(kRecColThreads) rec_cols_kernel(const __grid_c
 
 }  // namespace
 
-static cudaError_t launch_scan(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s) {
-    max_H = max_H < kRecMaxLine ? max_H : kRecMaxLine;
-    max_W = max_W < kRecMaxLine ? max_W : kRecMaxLine;
-    auto go = [&](auto k, int nlines, int len, int arrays) -> cudaError_t {
-        auto bytes = [&](int n) { return (size_t)kRecPairs * rec_pair_floats2(n, arrays) * sizeof(float2); };
-        const size_t smem = bytes(len);
-        cudaError_t e = allow_smem(k, bytes(kRecMaxLine));
+cudaError_t launch_recursive_scan(const RecursiveLaunch& L, int axis, int nimg, int lines, int len, cudaStream_t s) {
+    if (nimg <= 0) return cudaSuccess;
+    auto go = [&](auto k, int arrays) -> cudaError_t {
+        cudaError_t e = allow_smem(k, rec_smem_bytes(kRecMaxLine, arrays));
         if (e != cudaSuccess) return e;
-        const int nblk = (nlines + kRecLines - 1) / kRecLines;
-        k<<<(unsigned)(nimg * nblk), 32 * kRecPairs, smem, s>>>(L, nblk);
+        const int nblk = (lines + kRecLines - 1) / kRecLines;
+        k<<<(unsigned)(nimg * nblk), 32 * kRecPairs, rec_smem_bytes(len, arrays), s>>>(L, nblk);
         return cudaGetLastError();
     };
-    cudaError_t e;
-    if (L.mode == 0) {
-        if ((e = go(rec_rows_scan<true>, max_H, max_W, 3)) != cudaSuccess) return e;
-        if ((e = go(rec_cols_scan<0>, max_W, max_H, 3)) != cudaSuccess) return e;
-        return go(rec_cols_scan<1>, max_W, max_H, 2);
-    }
-    if ((e = go(rec_rows_scan<false>, max_H, max_W, 2)) != cudaSuccess) return e;
-    return go(rec_cols_scan<2>, max_W, max_H, 2);
+    if (axis == 1) return L.mode == 0 ? go(rec_rows_scan<true>, 3) : go(rec_rows_scan<false>, 2);
+    if (L.mode != 0) return go(rec_cols_scan<2>, 2);
+    const cudaError_t e = go(rec_cols_scan<0>, 3);
+    return e != cudaSuccess ? e : go(rec_cols_scan<1>, 2);
 }
 
-cudaError_t launch_recursive(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s) {
-    if (nimg <= 0 || max_H <= 0 || max_W <= 0) return cudaSuccess;
-    cudaError_t e = launch_scan(L, nimg, max_H, max_W, s);
-    if (e != cudaSuccess || rec_scans(max_H, max_W)) return e;
-    // images with a longer side
+cudaError_t launch_recursive_seq(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s) {
+    if (nimg <= 0) return cudaSuccess;
+    cudaError_t e;
     const size_t smem = (size_t)kRecRowWarps * kRecTileFloats * sizeof(float);
     if ((e = allow_smem(rec_rows_kernel<true>, smem)) != cudaSuccess) return e;
     if ((e = allow_smem(rec_rows_kernel<false>, smem)) != cudaSuccess) return e;
