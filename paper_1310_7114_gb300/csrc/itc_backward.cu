@@ -61,10 +61,12 @@ __device__ __forceinline__ void window_sums(const ImageDesc& D, float w0, float 
     int u = ua + lane / nv, v = va + lane % nv;
     float a = 0.f, d0 = 0.f, d1 = 0.f, d2 = 0.f;
     auto sums = [&](auto* h) {   // h: weights (null: ones); unconditional loads from clamped places
-        for (int p = lane; p < npos; p += 8 * 32) {
-            float x[8], du[8], dv[8], gl[8];
+        int p = lane;
+        auto block = [&](auto steps) {
+            constexpr int U = decltype(steps)::value;
+            float x[U], du[U], dv[U], gl[U];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < U; ++q) {
                 const size_t o = (size_t)min(u, ub) * D.pitch + v;
                 x[q] = h ? (float)__ldg(h + o) : 1.f;
                 gl[q] = ND == 3 ? (float)__ldg(reinterpret_cast<const unsigned char*>(D.data) + o) : 0.f;
@@ -78,7 +80,7 @@ __device__ __forceinline__ void window_sums(const ImageDesc& D, float w0, float 
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < U; ++q) {
                 const float dg = ND == 3 ? gl[q] - w2 : 0.f;
                 float e = du[q] * du[q] * c0 + dv[q] * dv[q] * c1;
                 if (ND == 3) e += dg * dg * c2;
@@ -89,7 +91,12 @@ __device__ __forceinline__ void window_sums(const ImageDesc& D, float w0, float 
                 d1 = fmaf(g, dv[q], d1);
                 if (ND == 3) d2 = fmaf(g, dg, d2);
             }
-        }
+            p += 32 * U;
+        };
+        // eight loads in flight, four where no more are left (10000 images of up to 16 px, whose boxes have
+        // 36 to 256 positions, M = 64: 568 us with eight throughout)
+        while (p - lane + 4 * 32 < npos) block(std::integral_constant<int, 8>());
+        if (p - lane < npos) block(std::integral_constant<int, 4>());
     };
     if (ND == 3) sums(D.weight);
     else if (D.dtype == ITC_U8) sums(reinterpret_cast<const unsigned char*>(D.data));
