@@ -189,6 +189,9 @@ void fill_desc(const itc_image* img, const itc_params* p, int M, ImageDesc* d) {
     d->sxx_tiles = (int)((long long)d->tiles_u * d->tiles_v * d->tiles_g);
 }
 
+long long bwd_strips(const ImageDesc& d) {
+    return d.ndim == 2 ? (long long)((d.H + kBwdStrip - 1) / kBwdStrip) * d.bwd_tiles_v : 0;
+}
 long long tiles_of(const ImageDesc& d) { return (long long)d.tiles_u * d.tiles_v * d.tiles_g; }
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
@@ -699,6 +702,7 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         d.bwd_tile_begin = bwd;
         bwd += d.bwd_tiles_u * d.bwd_tiles_v;
         h->max_bwd_tiles = std::max(h->max_bwd_tiles, d.bwd_tiles_u * d.bwd_tiles_v);
+        h->bwd_strips += bwd_strips(d);
         if (d.M > maxM) maxM = d.M;
         h->max_dim[0] = d.H > h->max_dim[0] ? d.H : h->max_dim[0];
         h->max_dim[1] = d.W > h->max_dim[1] ? d.W : h->max_dim[1];
@@ -1340,6 +1344,7 @@ static int backward_images(const PlanHeader* h, const void* plan_host, const voi
     L.img_status = v.status;
     if (whole) {
         L.bwd_order = reinterpret_cast<const int*>(pd + h->ints_off) + h->bwd_order_off;
+        L.strips = h->bwd_strips;
         return cuda_status(launch_backward(L, h->B, h->max_M, h->bwd_tiles, h->max_bwd_tiles, h->ndim_mask, s));
     }
     // an image range: its CTAs in image order
@@ -1353,6 +1358,7 @@ static int backward_images(const PlanHeader* h, const void* plan_host, const voi
         max_tiles = std::max(max_tiles, t);
         max_M = std::max(max_M, hd[b].M);
         ndim_mask |= 1 << hd[b].ndim;
+        L.strips += bwd_strips(hd[b]);
     }
     L.bwd_order = nullptr;
     L.img_base = b0;

@@ -255,9 +255,8 @@ __global__ void __launch_bounds__(kCodebookThreads, 1) bwd_codebook_kernel(const
 }
 
 constexpr int kPixWarps = 4;    // warps of a 2-D pixel CTA
-constexpr int kPixRows = 16, kPixCols = 64;   // a warp's tile
+constexpr int kPixRows = kBwdStrip;   // rows of a warp's tile
 constexpr int kPixSlots = 16;   // codebook vectors staged per turn
-constexpr int kPixStage = kPixRows + kPixCols;   // floats of one: a, then b
 
 // 2-D pixel pass.  The stamp S(x) = sum_k g(x - w_k) [x in box(round(w_k))] is separable:
 // g(x - w) = g_u(x_u - w_u) g_v(x_v - w_v) and the box is a product of two intervals, so for the vectors
@@ -270,6 +269,10 @@ constexpr int kPixStage = kPixRows + kPixCols;   // floats of one: a, then b
 // (64 x 64 tiles of a CTA with a barrier per phase: 113 us for 256 images of 512 x 512, 6.3 TB/s in 85 us now;
 // 589 and 464 us for 4096 ragged images).  Row pieces of 256 bytes: fields and gradients of ragged images start
 // anywhere in a 128-byte line, and with 32 x 32 tiles the shared lines cost 514 us.
+// COLS 16: where a batch has too few tiles for all warps, the chain of a warp over the vectors is the time of
+// the pass, and 16 x 16 tiles (4 x 2 per lane) make a vector's step shorter.  Every pixel adds the same products in
+// the same order (39 images of 16 x 16, 300 vectors, the whole backward: 62 us, 77 with 16 x 64 tiles).
+template <int COLS>
 __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const __grid_constant__ BackwardLaunch L) {
     // split CTAs per image: the warps take its tiles in turn
     const int split = L.split;
@@ -277,8 +280,11 @@ __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const _
     const ImageDesc& D = L.descs[img];
     if (D.ndim != 2) return;
     const int M = D.M, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int RB = COLS == 64 ? 8 : 4, CB = COLS == 64 ? 4 : 2;   // a lane's rows and columns of a tile
+    constexpr int STAGE = kPixRows + COLS;                             // floats of a staged vector: a, then b
+    static_assert(kPixRows / RB * (COLS / CB) == 32, "a lane's block");
     const int H = D.H, Wd = D.W, fpitch = D.fpitch, Ru = D.R[0], Rv = D.R[1];
-    const int tiles_v = (Wd + kPixCols - 1) / kPixCols, ntiles = tiles_v * ((H + kPixRows - 1) / kPixRows);
+    const int tiles_v = (Wd + COLS - 1) / COLS, ntiles = tiles_v * ((H + kPixRows - 1) / kPixRows);
     const int first = (int)(blockIdx.x % split) * kPixWarps;
     if (first >= ntiles) return;
     // the separable factors exp(-d^2 c) = 2^(-d^2 c log2 e), log2 e folded into the widths
@@ -290,7 +296,7 @@ __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const _
 
     extern __shared__ __align__(16) unsigned char bsm[];
     float4* rec = reinterpret_cast<float4*>(bsm);   // per vector: position and site along u and v
-    __shared__ __align__(16) float stage[kPixWarps][kPixSlots][kPixStage];
+    __shared__ __align__(16) float stage[kPixWarps][kPixSlots][STAGE];
     const float* Wk = L.W + D.w_off;
     for (int k = tid; k < M; k += blockDim.x) {
         const float w0 = Wk[k * 2], w1 = Wk[k * 2 + 1];
@@ -298,39 +304,45 @@ __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const _
     }
     __syncthreads();
 
-    static_assert(kPixSlots * kPixStage >= kPixRows * kPixCols, "a warp's stage holds a tile");
-    float(*st)[kPixStage] = stage[wid];
-    const int br = lane >> 4 << 3, bc = (lane & 15) << 2;   // a lane's 8 x 4 block of a tile
+    static_assert(kPixSlots * STAGE >= kPixRows * COLS, "a warp's stage holds a tile");
+    float(*st)[STAGE] = stage[wid];
+    const int br = lane / (COLS / CB) * RB, bc = lane % (COLS / CB) * CB;   // a lane's block of a tile
     const bool rows16 = (Wd & 3) == 0 && (reinterpret_cast<size_t>(gh) & 15) == 0;
+    using Piece = std::conditional_t<CB == 4, float4, float2>;
     for (int t = first + wid; t < ntiles; t += split * kPixWarps) {
-        const int u0 = t / tiles_v * kPixRows, v0 = (t - t / tiles_v * tiles_v) * kPixCols;
+        const int u0 = t / tiles_v * kPixRows, v0 = (t - t / tiles_v * tiles_v) * COLS;
         const int u = u0 + lane, v = v0 + lane, nrow = min(kPixRows, H - u0);
-        // this lane's 8 x 4 block of the field, loaded first so that its latency overlaps the stamp
-        float4 f[8];
+        // this lane's block of the field, loaded first so that its latency overlaps the stamp
+        union { Piece v; float e[CB]; } f[RB];
         {
-            const float* p = A + min(v0 + bc, fpitch - 4);
+            const float* p = A + min(v0 + bc, fpitch - CB);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) f[i] = __ldg(reinterpret_cast<const float4*>(p + (size_t)min(u0 + br + i, H - 1) * fpitch));
+            for (int i = 0; i < RB; ++i) f[i].v = __ldg(reinterpret_cast<const Piece*>(p + (size_t)min(u0 + br + i, H - 1) * fpitch));
         }
-        float2 acc[4][4];   // row pairs, columns
+        float2 acc[RB / 2][CB];   // row pairs, columns
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < RB / 2; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.f, 0.f);
         const float fu = (float)u, fv = (float)v;
         int ns = 0;
         auto add = [&] {
             __syncwarp();
 #pragma unroll 1
             for (int l = 0; l < ns; ++l) {
-                const float4 b = *reinterpret_cast<const float4*>(&st[l][kPixRows + bc]);
-                const float4 a0 = *reinterpret_cast<const float4*>(&st[l][br]), a1 = *reinterpret_cast<const float4*>(&st[l][br + 4]);
-                const float2 a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
-                const float bj[4] = {b.x, b.y, b.z, b.w};
+                union { Piece v; float e[CB]; } b;
+                b.v = *reinterpret_cast<const Piece*>(&st[l][kPixRows + bc]);
+                float2 a[RB / 2];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int i = 0; i < RB / 2; i += 2) {
+                    const float4 a4 = *reinterpret_cast<const float4*>(&st[l][br + 2 * i]);
+                    a[i] = make_float2(a4.x, a4.y);
+                    a[i + 1] = make_float2(a4.z, a4.w);
+                }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[i][j] = __ffma2_rn(a[i], make_float2(bj[j], bj[j]), acc[i][j]);
+                for (int j = 0; j < CB; ++j)
+#pragma unroll
+                    for (int i = 0; i < RB / 2; ++i) acc[i][j] = __ffma2_rn(a[i], make_float2(b.e[j], b.e[j]), acc[i][j]);
             }
             __syncwarp();
             ns = 0;
@@ -340,50 +352,67 @@ __global__ void __launch_bounds__(32 * kPixWarps, 5) bwd_pixels2d_kernel(const _
             if (base + lane < M) {
                 const float4 r = rec[base + lane];
                 const int r0 = __float_as_int(r.z), r1 = __float_as_int(r.w);
-                hit = r0 + Ru >= u0 && r0 - Ru < u0 + kPixRows && r1 + Rv >= v0 && r1 - Rv < v0 + kPixCols;
+                hit = r0 + Ru >= u0 && r0 - Ru < u0 + kPixRows && r1 + Rv >= v0 && r1 - Rv < v0 + COLS;
             }
             unsigned bal = __ballot_sync(0xffffffffu, hit);
             while (bal) {
                 const float4 r = rec[base + __ffs(bal) - 1];
                 bal &= bal - 1;
-                const float du = fu - r.x, dv = fv - r.y;
-                const float dv2 = (float)(v + 32) - r.y;
-                if (lane < kPixRows) st[ns][lane] = abs(u - __float_as_int(r.z)) <= Ru ? ex2_ftz(-(du * du) * l0) : 0.f;
-                st[ns][kPixRows + lane] = abs(v - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv * dv) * l1) : 0.f;
-                st[ns][kPixRows + 32 + lane] = abs(v + 32 - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv2 * dv2) * l1) : 0.f;
+                if constexpr (COLS == 16) {   // the rows' factors on the first lanes, the columns' on the others
+                    const bool row = lane < kPixRows;
+                    const int x = row ? u : v - kPixRows;
+                    const float d = (float)x - (row ? r.x : r.y);
+                    const int site = __float_as_int(row ? r.z : r.w);
+                    st[ns][lane] = abs(x - site) <= (row ? Ru : Rv) ? ex2_ftz(-(d * d) * (row ? l0 : l1)) : 0.f;
+                } else {
+                    const float du = fu - r.x, dv = fv - r.y;
+                    const float dv2 = (float)(v + 32) - r.y;
+                    if (lane < kPixRows) st[ns][lane] = abs(u - __float_as_int(r.z)) <= Ru ? ex2_ftz(-(du * du) * l0) : 0.f;
+                    st[ns][kPixRows + lane] = abs(v - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv * dv) * l1) : 0.f;
+                    st[ns][kPixRows + 32 + lane] = abs(v + 32 - __float_as_int(r.w)) <= Rv ? ex2_ftz(-(dv2 * dv2) * l1) : 0.f;
+                }
                 if (++ns == kPixSlots) add();
             }
         }
         if (ns) add();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < RB; ++i) {
             const float* q = &acc[i >> 1][0].x + (i & 1);
-            f[i] = make_float4(s1 * f[i].x - s2 * q[0], s1 * f[i].y - s2 * q[2], s1 * f[i].z - s2 * q[4], s1 * f[i].w - s2 * q[6]);
+#pragma unroll
+            for (int j = 0; j < CB; ++j) f[i].e[j] = s1 * f[i].e[j] - s2 * q[2 * j];
         }
         if (rows16) {
             float* out = gh + (size_t)(u0 + br) * Wd + v0 + bc;
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (v0 + bc < Wd && br + i < nrow) *reinterpret_cast<float4*>(out + (size_t)i * Wd) = f[i];
+            for (int i = 0; i < RB; ++i)
+                if (v0 + bc < Wd && br + i < nrow) *reinterpret_cast<Piece*>(out + (size_t)i * Wd) = f[i].v;
             continue;
         }
         // rows on any boundary: through the warp's shared memory, a row piece to each store
         float* tile = &st[0][0];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(tile + (br + i) * kPixCols + bc) = f[i];
+        for (int i = 0; i < RB; ++i) *reinterpret_cast<Piece*>(tile + (br + i) * COLS + bc) = f[i].v;
         __syncwarp();
-        float* out = gh + (size_t)u0 * Wd + v;
-        const bool in0 = v < Wd, in1 = v + 32 < Wd;
-        if (nrow == kPixRows) {
+        if constexpr (COLS == 16) {
 #pragma unroll
-            for (int i = 0; i < kPixRows; ++i, out += Wd) {
-                if (in0) out[0] = tile[i * kPixCols + lane];
-                if (in1) out[32] = tile[i * kPixCols + 32 + lane];
+            for (int i = 0; i < kPixRows; i += 2) {   // two rows at a time
+                const int r = i + (lane >> 4), c = lane & 15;
+                if (r < nrow && v0 + c < Wd) gh[(size_t)(u0 + r) * Wd + v0 + c] = tile[r * COLS + c];
             }
         } else {
-            for (int i = 0; i < nrow; ++i, out += Wd) {
-                if (in0) out[0] = tile[i * kPixCols + lane];
-                if (in1) out[32] = tile[i * kPixCols + 32 + lane];
+            float* out = gh + (size_t)u0 * Wd + v;
+            const bool in0 = v < Wd, in1 = v + 32 < Wd;
+            if (nrow == kPixRows) {
+#pragma unroll
+                for (int i = 0; i < kPixRows; ++i, out += Wd) {
+                    if (in0) out[0] = tile[i * COLS + lane];
+                    if (in1) out[32] = tile[i * COLS + 32 + lane];
+                }
+            } else {
+                for (int i = 0; i < nrow; ++i, out += Wd) {
+                    if (in0) out[0] = tile[i * COLS + lane];
+                    if (in1) out[32] = tile[i * COLS + 32 + lane];
+                }
             }
         }
         __syncwarp();
@@ -582,8 +611,16 @@ cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long
         kernel<<<(unsigned)(B * (long long)L2.split), threads, smem, s>>>(L2);
         e = cudaGetLastError();
     };
-    if (ndim_mask & 4)
-        launch(bwd_pixels2d_kernel, 32 * kPixWarps, sizeof(float4), 6, max_image_tiles);
+    if (ndim_mask & 4) {
+        // of 20 warps per SM; many vectors make the chain longer, few do not repay the shorter row pieces (244
+        // images of 64 x 64, 976 strips: with 2, 16, 64 and 300 vectors 20.5, 22.3, 29.5 and 76.9 us in strips and
+        // 21.6, 23.5, 29.9 and 67.7 in 16 x 16 tiles; 1952 strips, 300 vectors: 91 and 108)
+        static_assert(kBwdStrip == kPixRows && kBwdTileW == 64, "a strip is a warp's tile");
+        if (2 * L.strips <= (max_M > 64 ? 20LL : 10LL) * sms)
+            launch(bwd_pixels2d_kernel<16>, 32 * kPixWarps, sizeof(float4), 1, 4LL * max_image_tiles);
+        else
+            launch(bwd_pixels2d_kernel<64>, 32 * kPixWarps, sizeof(float4), 6, max_image_tiles);
+    }
     if (e == cudaSuccess && (ndim_mask & 8)) {   // list records, positions, sites, tile list
         constexpr size_t per_vector = 16 + 7 * sizeof(int);
         if (4 * pixel_tiles < 3LL * sms) launch(bwd_pixels3d_kernel<16>, kThreads, per_vector, 1, 16LL * max_image_tiles);

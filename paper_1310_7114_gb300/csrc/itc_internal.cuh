@@ -141,6 +141,7 @@ struct PlanHeader {
                                 // position (the launch of class c from list position p uses
                                 // list_off(c) + p)
     long long bwd_tiles;        // backward pixel tiles over all images
+    long long bwd_strips;       // and their strips (of the 2-D images)
     int max_bwd_tiles;          // most backward pixel tiles of one image
     int bwd_order_off;          // offset (ints) of the backward image order (B ints, most tiles first)
     int run_groups_off;         // offset (ints) of the iteration groups (kGroupInts ints each)
@@ -256,6 +257,7 @@ struct BackwardLaunch {
                                 // nullptr: images img_base, img_base + 1, ... in order
     int B;
     int split;                  // pixel-pass CTAs per image (set at launch)
+    long long strips;           // 16 x 64 strips of the launch's 2-D images
     int img_base;               // image of the first CTA (image ranges)
     const int* img_status;      // per-image status words of the fields pass, or nullptr
 };
@@ -289,6 +291,7 @@ struct SegmentLaunch {
 
 constexpr int kBwdTileH = 64;   // backward pixel tile: 64 rows x 64 columns
 constexpr int kBwdTileW = 64;
+constexpr int kBwdStrip = 16;   // rows of a strip, a warp's tile of the 2-D pass
 constexpr int kGridTileH2 = 64;   // fields tile height, 2-D (plain staging)
 constexpr int kGridTileH3 = 32;   // fields tile height, 3-D (one gray slice per tile)
 
