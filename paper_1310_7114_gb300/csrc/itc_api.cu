@@ -1136,7 +1136,7 @@ int itc_segment(const void* plan_host, const void* plan_dev, const float* W, sho
     L.labels = labels;
     L.split = 1;
     L.order = reinterpret_cast<const int*>(pd + h->ints_off) + h->bwd_order_off;
-    return cuda_status(launch_segment(L, h->B, h->max_M, h->max_bwd_tiles, h->kind_mask,
+    return cuda_status(launch_segment(L, h->B, h->max_M, h->max_bwd_tiles, h->max_dim[0], h->max_dim[1], h->kind_mask,
                                       reinterpret_cast<cudaStream_t>(stream)));
 }
 

@@ -332,8 +332,10 @@ cudaError_t launch_recursive_scan(const RecursiveLaunch& L, int axis, int nimg, 
 // both axes of images whose lines are filtered sequentially
 cudaError_t launch_recursive_seq(const RecursiveLaunch& L, int nimg, int max_H, int max_W, cudaStream_t s);
 cudaError_t launch_chamfer(const ChamferLaunch& L, int max_W, cudaStream_t s);
-// max_blocks: most 64 x 64 pixel blocks of one image; kinds: bit kSeg* for each kind of image in the plan
-cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int kinds, cudaStream_t s);
+// max_blocks: most 64 x 64 pixel blocks of one image; max_H, max_W: largest sides; kinds: bit kSeg* for each kind
+// of image in the plan
+cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int max_H, int max_W, int kinds,
+                           cudaStream_t s);
 cudaError_t launch_backward(const BackwardLaunch& L, int B, int max_M, long long pixel_tiles, int max_image_tiles,
                             int ndim_mask, cudaStream_t s);
 }  // namespace itc
