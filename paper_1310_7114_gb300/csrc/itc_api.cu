@@ -378,7 +378,7 @@ int rec_seq_side(const ClassInfo& ci, const ImageDesc* descs, const int* list) {
 // Microseconds with all images in one launch and now: 256 of 128 x 128 with one of 2048 x 2048 937 and 249
 // (sequential 1926), 47 of 500 x 500 with the same 595 and 352 (2165), 300 of 100 x 100 with 20 of 600 x 600 297
 // and 242 (655); 48 of 128 to 1024 px, in one launch, 555.  Splitting at twice the CTAs per SM made those 575.
-void rec_groups(ClassInfo& ci, const ImageDesc* descs, int* ints, int& io) {
+void rec_groups(const ClassInfo& ci, RecClass& rc, const ImageDesc* descs, int* ints, int& io) {
     const int* list = ints + ci.list_off;
     const int arrays = ci.self ? 2 : 3;
     auto step_of = [](int n) { return n <= 256 ? 0 : (n <= 512 ? 1 : (n <= 1024 ? 2 : 3)); };
@@ -400,7 +400,7 @@ void rec_groups(ClassInfo& ci, const ImageDesc* descs, int* ints, int& io) {
             ++c->n;
         }
         int ng = 0;
-        RecGroup* G = ci.rec_scan[axis];
+        RecGroup* G = rc.scan[axis];
         bool open = false;
         for (int k = 3; k >= 0; --k) {   // the longest lines first
             long long blocks = 0;
@@ -426,7 +426,7 @@ void rec_groups(ClassInfo& ci, const ImageDesc* descs, int* ints, int& io) {
                 G[ng - 1].lines = std::max(G[ng - 1].lines, c.lines);
             }
         }
-        ci.rec_ngroups[axis] = ng;
+        rc.ngroups[axis] = ng;
         for (int g = 0; g < ng; ++g) {
             G[g].off = io;
             for (int i = 0; i < ci.nimg; ++i) {
@@ -436,14 +436,14 @@ void rec_groups(ClassInfo& ci, const ImageDesc* descs, int* ints, int& io) {
             G[g].n = io - G[g].off;
         }
     }
-    ci.rec_seq = {io, 0, 0, 0};
+    rc.seq = {io, 0, 0, 0};
     for (int i = 0; i < ci.nimg; ++i) {
         const ImageDesc& d = descs[list[i]];
         if (!d.rec_seq) continue;
         ints[io++] = list[i];
-        ++ci.rec_seq.n;
-        ci.rec_seq.len = std::max(ci.rec_seq.len, d.W);
-        ci.rec_seq.lines = std::max(ci.rec_seq.lines, d.H);
+        ++rc.seq.n;
+        rc.seq.len = std::max(rc.seq.len, d.W);
+        rc.seq.lines = std::max(rc.seq.lines, d.H);
     }
 }
 
@@ -803,8 +803,12 @@ int itc_plan(int B, const itc_image* imgs, const int* M, const itc_params* p, in
         h->run_ngroups[nd - 2] = ng - nl;
     }
     const int count_ints = io;
-    for (int c = 0; c < h->ncls; ++c)
-        if (h->cls[c].recursive) rec_groups(h->cls[c], descs, ints, io);
+    for (int c = 0, nrec = 0; c < h->ncls; ++c) {
+        ClassInfo& ci = h->cls[c];
+        if (!ci.recursive) continue;
+        ci.rec = nrec++;   // (below kRecClasses: the keys of such classes differ in data type and pass alone)
+        rec_groups(ci, h->rec[ci.rec], descs, ints, io);
+    }
     h->nints = io;
     h->bwd_order_off = bwd_off;
     h->run_groups_off = run_off;
@@ -903,11 +907,12 @@ static int fields_range(const PlanHeader* h, const void* plan_host, const void* 
                 R.img_list = ints + g.off + q0;
                 return q1 - q0;
             };
-            int n = images(ci.rec_seq);
-            rc = cuda_status(launch_recursive_seq(R, n, ci.rec_seq.lines, ci.rec_seq.len, s));
+            const RecClass& C = h->rec[ci.rec];
+            int n = images(C.seq);
+            rc = cuda_status(launch_recursive_seq(R, n, C.seq.lines, C.seq.len, s));
             for (int axis = 1; axis >= 0; --axis)
-                for (int g = 0; g < ci.rec_ngroups[axis] && !rc; ++g) {
-                    const RecGroup& G = ci.rec_scan[axis][g];
+                for (int g = 0; g < C.ngroups[axis] && !rc; ++g) {
+                    const RecGroup& G = C.scan[axis][g];
                     n = images(G);
                     rc = cuda_status(launch_recursive_scan(R, axis, n, G.lines, G.len, s));
                 }

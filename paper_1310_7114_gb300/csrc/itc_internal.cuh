@@ -62,6 +62,13 @@ struct RecGroup {
     int off, n, len, lines;
 };
 constexpr int kRecGroups = 16;             // most per axis: four steps of line length, four of the number of lines
+// The launches of a recursive class: its scanned images by line length along u and along v, and those
+// filtered sequentially.
+struct RecClass {
+    RecGroup scan[2][kRecGroups], seq;
+    int ngroups[2];
+};
+constexpr int kRecClasses = 4;             // two data types, the fields and the self-overlap pass
 
 // One image as the kernels see it (device-resident inside a plan, or passed by value).
 struct ImageDesc {
@@ -111,8 +118,7 @@ struct ClassInfo {
     float tuned_ms;             // fields time of the class under the chosen configuration (0: untuned)
     int self;                   // self-overlap class: A at width s only, plain tiles
     int recursive;              // fields by recursive filtering (ITC_RECURSIVE); widths per image
-    RecGroup rec_scan[2][kRecGroups], rec_seq;   // its scanned images by line length along u and along v, and
-    int rec_ngroups[2];                          // those filtered sequentially
+    int rec;                    // its place in PlanHeader::rec
     int list_off;               // offset (ints) of this class's image list in the plan int area
     int prefix_off;             // offset (ints) of the class tile prefix (nimg + 1 ints)
     long long partial_base;     // first partial of the class
@@ -152,6 +158,7 @@ struct PlanHeader {
                                 // pass, then of the self-overlap pass
     long long pad_floats;       // sum H*fpitch (padded per-pixel layout)
     int has_recursive;          // some class computes its fields by recursion
+    RecClass rec[kRecClasses];
     ClassInfo cls[kMaxClasses];
 };
 
