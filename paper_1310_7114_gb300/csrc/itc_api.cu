@@ -98,10 +98,14 @@ void make_rec_coef(const float* sigma, const int* side, RecCoef* rc) {
             const double b = kRecDecay[t] / (double)sigma[a], ang = kRecOmega[t] / (double)sigma[a];
             rc->zr[a][t] = (float)(exp(-b) * cos(ang));
             rc->zi[a][t] = (float)(exp(-b) * sin(ang));
-            for (int k = 0; k < 5; ++k) {
-                const double n = (double)((side[a] + 31) / 32 * (1LL << k));
-                rc->pr[a][t][k] = (float)(exp(-b * n) * cos(ang * n));
-                rc->pi[a][t][k] = (float)(exp(-b * n) * sin(ang * n));
+            const double n = (double)((side[a] + 31) / 32), mag = exp(-b * n);
+            double re = mag * cos(ang * n), im = mag * sin(ang * n);
+            for (int k = 0; k < 5; ++k) {   // z^n, squared from one to the next
+                rc->pr[a][t][k] = (float)re;
+                rc->pi[a][t][k] = (float)im;
+                const double r2 = re * re - im * im;
+                im *= 2 * re;
+                re = r2;
             }
         }
     for (int t = 0; t < 2; ++t) {
@@ -180,7 +184,8 @@ void fill_desc(const itc_image* img, const itc_params* p, int M, ImageDesc* d) {
         for (int i = 0; i < 3; ++i) sw[i] = i < img->ndim ? self_width(p, i) : 1.f;
         const int side[2] = {img->H, img->W};
         make_rec_coef(p->sigma, side, &d->rc);
-        make_rec_coef(sw, side, &d->rc_self);
+        if (sw[0] == p->sigma[0] && sw[1] == p->sigma[1]) d->rc_self = d->rc;
+        else make_rec_coef(sw, side, &d->rc_self);
     }
     d->self_tiles_u = d->tiles_u;
     d->self_off = -1;
