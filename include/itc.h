@@ -339,7 +339,7 @@ int itc_run_staged(const void* plan_host, const void* plan_dev, const void* host
  * fastest on this GPU for this batch: the rows of output per tile (128, 64 or 32, i.e. how much
  * of the R-wide halo the row pass recomputes), the number of persistent CTAs per SM (1 or as many
  * as fit), and the input staging (tensor-memory-accelerator tiles, where the image rows are
- * 16-byte aligned, or plain loads).  Each candidate is timed with CUDA events over `reps`
+ * 16-byte aligned, or copies by the threads).  Each candidate is timed with CUDA events over `reps`
  * launches (after one untimed launch) on `stream`; the choice is stored in the host plan and
  * the updated plan is copied to plan_dev (synchronously).  Results of later calls do not
  * depend on the choice except for the summation order of S_XX (fields are identical).
@@ -351,7 +351,8 @@ int itc_autotune(void* plan_host, void* plan_dev, void* ws, size_t ws_bytes, int
 /*
  * itc_plan_configure -- set the fields-pass configuration of class c by hand (what itc_autotune
  * chooses): staging 1 = tensor tiles with tile_h 64 output rows (or 32 or 128 for radii 6, 9 and 12),
- * staging 0 = thread loads (any row alignment) with the fixed tile height of the lattice dimension (64 in 2-D, 32 in 3-D; pass it);
+ * staging 0 = copies by the threads (any row alignment; plain loads where no tiles are compiled for
+ * the radius) with the fixed tile height of the lattice dimension (64 in 2-D, 32 in 3-D; pass it);
  * grid_per_sm = persistent CTAs per SM (0 = as many as fit, else 1..64).  Updates the host
  * plan and copies it to plan_dev (synchronously on `stream`).  Errors: ITC_ERR_INVALID_ARG,
  * ITC_ERR_UNSUPPORTED (tensor tiles for a class whose images or radius cannot use them, or a
@@ -366,9 +367,10 @@ int itc_plan_classes(const void* plan_host);
 /*
  * itc_plan_class -- the configuration of class c (host-only): lattice dimension, sigma, output
  * rows per fields tile, persistent CTAs per SM (0 = as many as fit), staging (1 = tensor tiles,
- * 0 = plain loads, 2 = the extra pass that computes the field of h at the width of V(X) for
- * images whose sigma_self differs from sigma: plain loads, A only, 3 = recursive filtering,
- * ITC_RECURSIVE), number of images and the
+ * 0 = copies by the threads, or plain loads where no tiles are compiled for the radius, 2 = the
+ * extra pass that computes the field of h at the width of V(X) for images whose sigma_self differs
+ * from sigma: A only, staged as the image's rows allow, 3 = recursive filtering, ITC_RECURSIVE),
+ * number of images and the
  * tuned fields time in ms (0 if not tuned).  Any output pointer may be NULL.
  * Errors: ITC_ERR_INVALID_ARG.
  */

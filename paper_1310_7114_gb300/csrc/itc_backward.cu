@@ -10,7 +10,7 @@
 // window sums around round(w_k) read directly from the image (kernel evaluated at the real w_k, one
 // warp per k), the M x M sums s_k, E_k (one thread per k), S_XW, S_WW, grad_W and two per-image
 // scalars for kernel 2.
-// Kernel 2 (per dimension; 16 x 64 pixel tiles of a warp in 2-D, 32 x 32 or 16 x 16 of a CTA in 3-D): the codebooks
+// Kernel 2 (per dimension; 16 x 64 or 16 x 16 pixel tiles of a warp in 2-D, 32 x 32 or 16 x 16 of a CTA in 3-D): the codebooks
 // whose box meets a tile are taken in k order (ballots), their Gaussians are stamped onto the tile in
 // that order -- the transposed form of the gather in the forward update -- and every pixel
 // combines the stored field A with the stamp.
