@@ -20,6 +20,7 @@
 // 128, 84 Mpx): 0.67 -> 0.18 ms; before, every 16 x 16 tile listed from the whole codebook, with or
 // without data, and each pixel ran through its list in integers.
 #include <algorithm>
+#include <type_traits>
 
 #include "itc_internal.cuh"
 
@@ -29,7 +30,7 @@ namespace {
 constexpr int kSegBlock = 64;            // block side
 constexpr int kSegTile = 16;             // tile side (8 x 32 tiles list 1.4 times the codebooks)
 constexpr int kSegRows = kSegTile / 2;   // rows per lane
-constexpr int kSegThreads = 128;         // most threads of a CTA
+constexpr int kSegWarps = 4;             // most warps of a CTA
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float site_round(float x, int n) {
@@ -95,11 +96,11 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
     const int H = D.H, Wd = D.W, G = D.G, pitch = D.pitch, M = D.M;
     const unsigned char* gray = reinterpret_cast<const unsigned char*>(D.data);   // 3-D
     const int blocks_v = (Wd + kSegBlock - 1) / kSegBlock, nblocks = blocks_v * ((H + bh - 1) / bh);
+    // up to 32 vectors are a step of the tile's own list, and an image of one tile needs no other
+    const bool tile_only = M <= 32 || (H <= kSegTile && Wd <= kSegTile);
     for (int t = t0; t < nblocks; t += step) {
         const int ub = (t / blocks_v) * bh, vb = (t % blocks_v) * kSegBlock;
-        // the block's list is made when a tile needs it; up to 32 vectors are a step of the tile's own list,
-        // and a block of one tile needs no other
-        const bool tile_only = M <= 32 || (min(bh, H - ub) <= kSegTile && Wd - vb <= kSegTile);
+        // the block's list is made when a tile needs it
         int nb = tile_only ? M : -1;
         const unsigned short* from = tile_only ? nullptr : S.block;
         for (int half = 0; half < 2; ++half) {
@@ -202,13 +203,13 @@ __device__ __forceinline__ void segment_blocks(const ImageDesc& D, const T* data
 
 // split CTAs per image: their warps share out its blocks.  KIND: the images of the launch, bytes, weights or
 // gray (others return).
-template <int KIND>
-__global__ void __launch_bounds__(kSegThreads, KIND == kSegGray ? 4 : 5) segment_kernel(const __grid_constant__ SegmentLaunch L) {
+template <int KIND, int NW>
+__global__ void __launch_bounds__(32 * NW, (KIND == kSegGray ? 4 : 5) * kSegWarps / NW) segment_kernel(const __grid_constant__ SegmentLaunch L) {
     const int img = __ldg(L.order + blockIdx.x / L.split), part = blockIdx.x % L.split;
     const ImageDesc& D = L.descs[img];
     constexpr int nd = KIND == kSegGray ? 3 : 2;
     if ((D.ndim == 3 ? kSegGray : (D.dtype == ITC_U8 ? kSegBytes : kSegWeights)) != KIND) return;
-    const int M = D.M, tid = threadIdx.x, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int M = D.M, tid = threadIdx.x, wid = tid >> 5, nw = NW;
     const int blocks = D.bwd_tiles_u * D.bwd_tiles_v;
     static_assert(kSegBlock == kBwdTileH && kSegBlock == kBwdTileW, "blocks are the backward's tiles");
     // strips of 16 rows where there are few blocks for the image's warps: 770 images of up to 67 px with 8
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(kSegThreads, KIND == kSegGray ? 4 : 5) segment
     S.block = reinterpret_cast<unsigned short*>(S.site_g + M) + 2 * wid * M;
     S.tile = S.block + M;
     const float* Wk = L.W + D.w_off;
-    for (int k = tid; k < M; k += blockDim.x) {
+    for (int k = tid; k < M; k += 32 * NW) {
         S.site[k] = make_float2(site_round(Wk[k * nd], D.H), site_round(Wk[k * nd + 1], D.W));
         S.site_g[k] = nd == 3 ? site_round(Wk[k * nd + nd - 1], D.G) : 0.f;
     }
@@ -239,26 +240,23 @@ __global__ void __launch_bounds__(kSegThreads, KIND == kSegGray ? 4 : 5) segment
     else segment_blocks<2>(D, reinterpret_cast<const float*>(D.data), S, out, t0, step, bh, q);
 }
 
-template <int KIND>
-cudaError_t launch_kind(const SegmentLaunch& L, int B, int max_M, int max_blocks, int max_strips, cudaStream_t s) {
-    // no more warps than the largest image has strips: a CTA's idle warps would keep others off the SM (10000
-    // gray images of 4 to 16 px, 64 vectors: 189 us with four warps, 83 with one)
-    const int nw = std::min(kSegThreads / 32, max_strips);
-    auto bytes = [](size_t M, int warps) { return M * (3 * sizeof(float) + 2 * warps * sizeof(unsigned short)); };
-    const size_t smem = bytes(max_M, nw);
-    cudaError_t e = allow_smem(segment_kernel<KIND>, bytes(ITC_MAX_M, kSegThreads / 32));
+template <int KIND, int NW>
+cudaError_t launch_kind(const SegmentLaunch& L, int B, int max_M, int max_blocks, cudaStream_t s) {
+    constexpr size_t per_vector = 3 * sizeof(float) + 2 * NW * sizeof(unsigned short);
+    const size_t smem = (size_t)max_M * per_vector;
+    cudaError_t e = allow_smem(segment_kernel<KIND, NW>, ITC_MAX_M * per_vector);
     if (e != cudaSuccess) return e;
     // a large image is shared out over several CTAs, eight blocks a warp (four: 5 % slower, more CTAs stage
     // the sites).  A batch that does not fill the GPU (152 SMs, five CTAs each) takes a block a warp, two if
     // that makes many CTAs, and as few as a strip while it leaves SMs without work (300 ragged images 86 ->
     // 64 us, 42 of 500 px with 327 vectors 75 -> 49, one of 300 px 19 -> 7).
-    const int slots = 152 * 5;
+    constexpr int nw = NW, slots = 152 * 5;
     auto ctas = [&](int blocks_per_warp) { return (max_blocks + blocks_per_warp * nw - 1) / (blocks_per_warp * nw); };
     SegmentLaunch L2 = L;
     if (B >= slots) L2.split = ctas(8);
     else if ((long long)B * ctas(1) >= 4 * slots) L2.split = ctas(2);
     else L2.split = std::max(ctas(1), std::min((kSegBlock / kSegTile * max_blocks + nw - 1) / nw, slots / B));
-    segment_kernel<KIND><<<(unsigned)(B * L2.split), 32 * nw, smem, s>>>(L2);
+    segment_kernel<KIND, NW><<<(unsigned)(B * L2.split), 32 * NW, smem, s>>>(L2);
     return cudaGetLastError();
 }
 
@@ -267,11 +265,18 @@ cudaError_t launch_kind(const SegmentLaunch& L, int B, int max_M, int max_blocks
 cudaError_t launch_segment(const SegmentLaunch& L, int B, int max_M, int max_blocks, int max_H, int max_W, int kinds, cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
     static_assert(ITC_MAX_M <= 65535, "16-bit lists");
-    const int strips = (max_H + kSegTile - 1) / kSegTile * ((max_W + kSegBlock - 1) / kSegBlock);   // or more
+    // images of one strip: a warp each, three idle ones would keep others off the SM (10000 gray images of 4 to 16
+    // px, 64 vectors: 189 us with four warps, 83 with one)
+    const bool one = max_H <= kSegTile && max_W <= kSegBlock;
     cudaError_t e = cudaSuccess;
-    if (kinds & (1 << kSegBytes)) e = launch_kind<kSegBytes>(L, B, max_M, max_blocks, strips, s);
-    if (e == cudaSuccess && (kinds & (1 << kSegWeights))) e = launch_kind<kSegWeights>(L, B, max_M, max_blocks, strips, s);
-    if (e == cudaSuccess && (kinds & (1 << kSegGray))) e = launch_kind<kSegGray>(L, B, max_M, max_blocks, strips, s);
+    auto launch = [&](auto kind) {
+        constexpr int K = decltype(kind)::value;
+        if (e == cudaSuccess && (kinds & (1 << K)))
+            e = one ? launch_kind<K, 1>(L, B, max_M, max_blocks, s) : launch_kind<K, kSegWarps>(L, B, max_M, max_blocks, s);
+    };
+    launch(std::integral_constant<int, kSegBytes>());
+    launch(std::integral_constant<int, kSegWeights>());
+    launch(std::integral_constant<int, kSegGray>());
     return e;
 }
 
