@@ -38,10 +38,10 @@ FALLBACK_HBM_GBS = 6800.0
 # profiles/fields3d_kernel_c5_gray3d.md), valid only for the kernel source it was taken on
 # (sha256 prefix below); scaled to a launch by its site count (pixels, or voxels of the 3-D lattice).
 FIELDS_TRAFFIC = {
-    "c3": {"bytes_per_site": 968.86e6 / 86358723, "source_sha256": "2219d1a8248e79c7",
+    "c3": {"bytes_per_site": 969.22e6 / 86358723, "source_sha256": "b4e07329e6363145",
            "source": "paper_1310_7114_gb300/csrc/itc_fields_tma.cuh",
            "note": "ncu dram bytes of the 1024-image capture scaled by pixels (profiles/fields_tma_kernel_c3_1024.md)"},
-    "c5": {"bytes_per_site": (0.27e6 + 206.93e6) / 16777216, "source_sha256": "6eedaafde8ac4a48",
+    "c5": {"bytes_per_site": (0.21e6 + 206.58e6) / 16777216, "source_sha256": "2e6cf066545e002d",
            "source": "paper_1310_7114_gb300/csrc/itc_fields3d.cu",
            "note": "ncu dram bytes of one launch (profiles/fields3d_kernel_c5_gray3d.md)"},
 }
